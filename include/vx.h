@@ -177,13 +177,15 @@ vx_status vx_filter(vx_ctx *ctx, const vx_pred *preds, int32_t n_preds, uint64_t
  * behaviour:
  *   - n_rows above 67,108,864 (2^26) returns VX_E_INVAL;
  *   - count > cap returns VX_E_CAPACITY after writing the first cap ids;
+ *   - the call's blocks wait for one another's counts; a wait that runs out
+ *     (each is bounded) returns VX_E_TIMEOUT;
  *   - the first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress with that device current) and keeps it for the
  *     life of the process, so the device must not be reset (cudaDeviceReset)
  *     between calls;
  *   - every call shares the one array, so calls whose work overlaps on the
- *     GPU (other streams, other host threads) race and give wrong results:
- *     serialise them. */
+ *     GPU (other streams, other host threads) race and give wrong results or
+ *     VX_E_TIMEOUT: serialise them. */
 vx_status vx_filter_device_static(const int32_t *const *cols, int32_t n_cols, const vx_pred *preds,
                                   int32_t n_preds, uint64_t n_rows, uint64_t row0, uint64_t *out_rows,
                                   uint64_t cap, uint64_t *out_count, void *stream);
