@@ -528,7 +528,8 @@ typedef struct {
   double ms_sample, ms_train, ms_build, ms_probe, ms_kernel, ms_total;
   double ms_probe_kernel;  /* device time of the probe kernels alone (CUDA events); every probe key
                               is looked up in exactly one partition */
-  uint64_t bytes_d2h;      /* RADIX: clustered chunks and boundary arrays stored to host memory */
+  uint64_t bytes_d2h;      /* RADIX: clustered chunks and boundary arrays stored to host memory (0 when
+                              both clustered tables fitted the arena and stayed there) */
   uint32_t algorithm;      /* VX_JOIN_* that ran */
   uint32_t ranges;         /* RADIX: group ranges of the join pass */
   double ms_partition;     /* RADIX: wall time of the partition passes of both tables */
@@ -540,9 +541,10 @@ typedef struct {
  * into n_partitions key ranges; for each range an open-addressing table is
  * built in HBM from the streamed build side and the streamed probe side
  * probes it (Section 5.3 executor for every stream).  RADIX (opts->algorithm):
- * the paper's radix-partitioned join (see VX_JOIN_RADIX); its host
+ * the paper's radix-partitioned join (see VX_JOIN_RADIX); its clustered
+ * chunks stay in the arena when they fit it, else they go through host
  * intermediates (16 B per build row, 12 B per probe row, 4 (2^bits + 1) B per
- * chunk) are allocated for the call.  Returns VX_E_DUPKEY if a build key
+ * chunk) allocated for the call.  Returns VX_E_DUPKEY if a build key
  * repeats. */
 vx_status vx_join(vx_ctx *ctx, int32_t build_key, int32_t build_payload, int32_t probe_key, const vx_join_opts *opts,
                   vx_join_result *out);
