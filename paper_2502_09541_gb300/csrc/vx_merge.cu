@@ -707,7 +707,7 @@ vx_status merge_sort_plan(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
       VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
       ss.bytes_h2d += es.bytes_h2d;
       ss.bytes_d2h += es.bytes_d2h;
-      ss.kernel_launches += es.kernel_launches * 37;  // radix sort (35), fences, publish
+      ss.kernel_launches += es.kernel_launches * 12;  // radix sort (10), fences, publish
       ss.ms_sort_kernel += es.ms_kernel;
       ss.radix_pass_pairs += rp.pass_pairs;
     }

@@ -6,15 +6,15 @@
 //
 // Range partition = upsweep (per-tile digit histograms) -> row scan (per
 // digit, exclusive over tiles) -> totals scan (exclusive over digits: the
-// boundary array of Section 6.2.1) -> downsweep (stable scatter).  An LSD sort
-// pass is one scatter kernel: the global digit offsets of all eight passes
-// come from one histogram read of the keys, and each tile finds the count of
-// its digits in the tiles before it by decoupled look-back (tiles take
-// tickets in launch order, publish their counts, then their inclusive
-// prefixes; every wait is bounded and sets the error word when it gives up).
-// Ranking inside a tile is warp-contiguous: warp w owns 512 consecutive pairs
-// and processes them in 16 rounds of 32; __match_any_sync groups equal digits
-// of a round, so pairs keep their input order (stability).
+// boundary array of Section 6.2.1) -> scatter (stable).  An LSD sort pass is
+// one scatter kernel: the global digit offsets of all passes come from one
+// histogram read of the keys, and each tile finds the count of its digits in
+// the tiles before it by decoupled look-back (tiles take tickets in launch
+// order, publish their counts, then their inclusive prefixes; every wait is
+// bounded and sets the error word when it gives up).  Ranking inside a tile is
+// warp-contiguous: warp w owns 512 consecutive pairs and processes them in 16
+// rounds of 32; the lanes of a round with equal digits find one another, so
+// pairs keep their input order (stability).
 //
 // Double buffer: `cur[pass]` (device) says which of (A, B) holds the input of
 // LSD pass `pass`; a pass whose digit is constant over all pairs is skipped on

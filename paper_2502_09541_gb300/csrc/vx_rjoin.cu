@@ -686,7 +686,7 @@ vx_status radix_join_resident(vx_ctx *ctx, const Column *bk, const Column *bp, c
     ExecStats es;
     VX_TRY(run_pipeline(ctx, pp, &es));
     res.bytes_h2d += es.bytes_h2d;
-    res.kernel_launches += es.kernel_launches * (pp.npass + 6);
+    res.kernel_launches += es.kernel_launches * (pp.npass + 5);
     res.ms_kernel += es.ms_kernel;
   }
   res.ms_partition = res.ms_build = now_ms() - tp;
@@ -842,7 +842,7 @@ vx_status radix_join(vx_ctx *ctx, const Column *bk, const Column *bp, const Colu
     VX_TRY(run_pipeline(ctx, pp, &es));
     res.bytes_h2d += es.bytes_h2d;
     res.bytes_d2h += es.bytes_d2h;
-    res.kernel_launches += es.kernel_launches * (npass + 12);
+    res.kernel_launches += es.kernel_launches * (npass + 9);
     res.ms_kernel += es.ms_kernel;
   }
   res.ms_partition = now_ms() - tp;

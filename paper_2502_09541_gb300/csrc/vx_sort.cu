@@ -35,10 +35,8 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return m;
 }
 
-// digit of a key: an LSD byte (kRange = false) or the number of splitters <= key
-template <bool kRange>
-__device__ __forceinline__ uint32_t key_digit(uint64_t k, int shift, const uint64_t *s_spl, int n_spl) {
-  if (!kRange) return (uint32_t)(k >> shift) & 0xFFu;
+// partition of a key: the number of splitters <= key
+__device__ __forceinline__ uint32_t key_range(uint64_t k, const uint64_t *s_spl, int n_spl) {
   int lo = 0, hi = n_spl;
   while (lo < hi) {
     int mid = (lo + hi) >> 1;
@@ -48,26 +46,20 @@ __device__ __forceinline__ uint32_t key_digit(uint64_t k, int shift, const uint6
   return (uint32_t)lo;
 }
 
-template <bool kRange>
-__global__ void __launch_bounds__(kRxThreads) rx_upsweep(RadixBufs b, const RadixState *st, int pass, uint64_t n,
-                                                         int shift, const uint64_t *spl, int n_spl, uint32_t *hist,
+__global__ void __launch_bounds__(kRxThreads) rx_upsweep(const uint64_t *__restrict__ keys, uint64_t n,
+                                                         const uint64_t *spl, int n_spl, uint32_t *hist,
                                                          uint32_t ntiles) {
-  if (!kRange && st->skip[pass]) return;
   __shared__ uint32_t wcnt[kRxWarps][kRxDigits];
   __shared__ uint64_t s_spl[kRxDigits];
-  const int c = kRange ? 0 : st->cur[pass];
-  const uint64_t *keys = b.keys[c];
   for (int i = threadIdx.x; i < kRxWarps * kRxDigits; i += blockDim.x) (&wcnt[0][0])[i] = 0;
-  if (kRange)
-    for (int i = threadIdx.x; i < n_spl; i += blockDim.x) s_spl[i] = spl[i];
+  for (int i = threadIdx.x; i < n_spl; i += blockDim.x) s_spl[i] = spl[i];
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint64_t wbase = (uint64_t)blockIdx.x * kRxTile + (uint64_t)w * (32 * kRxItems);
 #pragma unroll 4
   for (int r = 0; r < kRxItems; ++r) {
     const uint64_t i = wbase + (uint64_t)r * 32 + lane;
-    const uint32_t d = i < n ? key_digit<kRange>(keys[i], shift, s_spl, n_spl) : kRxInvalid;
-    if (d != kRxInvalid) atomicAdd(&wcnt[w][d], 1u);  // counting needs no order
+    if (i < n) atomicAdd(&wcnt[w][key_range(keys[i], s_spl, n_spl)], 1u);  // counting needs no order
   }
   __syncthreads();
   for (int d = threadIdx.x; d < kRxDigits; d += blockDim.x) {
@@ -78,9 +70,7 @@ __global__ void __launch_bounds__(kRxThreads) rx_upsweep(RadixBufs b, const Radi
 }
 
 // block d: exclusive scan of hist[d][0..ntiles) in place; row total -> totals[d]
-__global__ void __launch_bounds__(1024) rx_scan_rows(uint32_t *hist, uint32_t ntiles, RadixState *st,
-                                                     const int pass, const bool check_skip) {
-  if (check_skip && st->skip[pass]) return;
+__global__ void __launch_bounds__(1024) rx_scan_rows(uint32_t *hist, uint32_t ntiles, RadixState *st) {
   __shared__ uint32_t wsum[32];
   __shared__ uint64_t carry;
   uint32_t *row = hist + (uint64_t)blockIdx.x * ntiles;
@@ -114,22 +104,13 @@ __global__ void __launch_bounds__(1024) rx_scan_rows(uint32_t *hist, uint32_t nt
   if (threadIdx.x == 0) st->totals[blockIdx.x] = carry;
 }
 
-// one block of 256 threads: digit bases (exclusive scan of totals, base[256] =
-// n); for LSD passes, a digit holding all n pairs marks the pass skipped and
-// the double-buffer marker advances only for executed passes
-__global__ void __launch_bounds__(kRxDigits) rx_scan_totals(RadixState *st, int pass, uint64_t n, bool lsd) {
+// one block of 256 threads: partition starts (exclusive scan of totals,
+// base[256] = n)
+__global__ void __launch_bounds__(kRxDigits) rx_scan_totals(RadixState *st, uint64_t n) {
   __shared__ uint64_t s[kRxDigits];
-  __shared__ int any_full;
   const int d = threadIdx.x;
-  if (lsd && st->skip[pass]) {  // decided by the digit-histogram prepass
-    if (d == 0) st->cur[pass + 1] = st->cur[pass];
-    return;
-  }
-  if (d == 0) any_full = 0;
-  __syncthreads();
   const uint64_t t = st->totals[d];
   s[d] = t;
-  if (t == n) any_full = 1;
   __syncthreads();
   for (int off = 1; off < kRxDigits; off <<= 1) {
     uint64_t y = d >= off ? s[d - off] : 0;
@@ -139,39 +120,60 @@ __global__ void __launch_bounds__(kRxDigits) rx_scan_totals(RadixState *st, int 
   }
   st->base[d] = s[d] - t;
   if (d == 0) st->base[kRxDigits] = n;
-  if (lsd && d == 0) {
-    st->skip[pass] = any_full;
-    st->cur[pass + 1] = any_full ? st->cur[pass] : 1 - st->cur[pass];
-  }
 }
 
-// full-range histogram of all eight key bytes in one read: marks constant
-// digits so that their passes are skipped (upsweep, scan and scatter)
-__global__ void __launch_bounds__(kRxThreads) rx_byte_hist(const RadixBufs b, uint64_t n, unsigned long long *bh) {
-  __shared__ uint32_t h[8][kRxDigits];
-  for (int i = threadIdx.x; i < 8 * kRxDigits; i += blockDim.x) (&h[0][0])[i] = 0;
+// histograms of the low npass key bytes in one read (constant digits are
+// skipped later)
+template <int kP>
+__global__ void __launch_bounds__(kRxThreads) rx_byte_hist(const uint64_t *__restrict__ keys, uint64_t n,
+                                                           unsigned long long *bh) {
+  __shared__ uint32_t h[kP][kRxDigits];
+  for (int i = threadIdx.x; i < kP * kRxDigits; i += blockDim.x) (&h[0][0])[i] = 0;
   __syncthreads();
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t k = b.keys[0][i];
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    uint64_t k[4];
 #pragma unroll
-    for (int p = 0; p < 8; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 0xFF], 1u);
+    for (int u = 0; u < 4; ++u) k[u] = keys[i + u * stride];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int p = 0; p < kP; ++p) atomicAdd(&h[p][(k[u] >> (8 * p)) & 0xFF], 1u);
   }
+  for (; i < n; i += stride)
+#pragma unroll
+    for (int p = 0; p < kP; ++p) atomicAdd(&h[p][(keys[i] >> (8 * p)) & 0xFF], 1u);
   __syncthreads();
-  for (int i = threadIdx.x; i < 8 * kRxDigits; i += blockDim.x)
+  for (int i = threadIdx.x; i < kP * kRxDigits; i += blockDim.x)
     if ((&h[0][0])[i]) atomicAdd(&bh[i], (unsigned long long)(&h[0][0])[i]);
 }
 
-__global__ void rx_init_state(RadixState *st, const unsigned long long *bh, uint64_t n, uint32_t spin_limit) {
-  const int p = threadIdx.x;  // 8 threads
-  if (p == 0) {
-    st->cur[0] = 0;
-    st->err = 0;
-    st->spin_limit = spin_limit;
+// one block of 256 threads per LSD pass: exclusive scan of the pass's digit
+// histogram (the global position of each digit's first pair) and whether one
+// digit holds all n pairs (the pass is skipped)
+__global__ void __launch_bounds__(kRxDigits) rx_init(RadixState *st, const unsigned long long *bh, uint64_t *bases,
+                                                     uint64_t n, uint32_t spin_limit) {
+  __shared__ uint64_t wsum[kRxDigits / 32];
+  const int p = blockIdx.x, d = threadIdx.x, lane = d & 31, w = d >> 5;
+  const uint64_t t = bh[p * kRxDigits + d];
+  uint64_t x = t;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
   }
-  if (p < 8) {
-    int full = 0;
-    for (int d = 0; d < kRxDigits; ++d) full |= bh[p * kRxDigits + d] == n;
+  if (lane == 31) wsum[w] = x;
+  const int full = __syncthreads_or(t == n);
+  for (int q = 0; q < w; ++q) x += wsum[q];
+  bases[p * kRxDigits + d] = x - t;
+  if (d == 0) {
     st->skip[p] = full;
+    if (p == 0) {
+      st->cur[0] = 0;
+      st->err = 0;
+      st->spin_limit = spin_limit;
+    }
   }
 }
 
@@ -198,57 +200,25 @@ __device__ __forceinline__ uint64_t rx_status_word(uint64_t flag, int pass, uint
   return flag | (uint64_t)pass << 59 | value;
 }
 
-// 8 blocks x 256 threads: exclusive scan of each digit histogram = the global
-// position of each digit's first pair in every LSD pass
-__global__ void __launch_bounds__(kRxDigits) rx_init_bases(const unsigned long long *bh, uint64_t *bases) {
-  __shared__ uint64_t s[kRxDigits];
-  const int p = blockIdx.x, d = threadIdx.x;
-  const uint64_t t = bh[p * kRxDigits + d];
-  s[d] = t;
-  __syncthreads();
-  for (int off = 1; off < kRxDigits; off <<= 1) {
-    const uint64_t y = d >= off ? s[d - off] : 0;
-    __syncthreads();
-    s[d] += y;
-    __syncthreads();
-  }
-  bases[p * kRxDigits + d] = s[d] - t;
-}
-
 // Stable scatter of one tile: rank every pair inside its warp (match_any over
 // 16 rounds of 32 consecutive pairs), regroup the tile by digit in shared
 // memory, then write each digit's run with consecutive threads on consecutive
 // output positions, so stores leave the SM as contiguous runs.
-// kOneSweep (LSD passes): the tile is the block's ticket, and its digit offsets
-// come from the one-read histogram (bases) plus a look-back over the status
-// words of the tiles before it; otherwise the tile is blockIdx.x and its
-// offsets come from the scanned per-tile histograms.
-template <bool kRange, bool kOneSweep>
-__global__ void __launch_bounds__(kRxThreads, 2) rx_downsweep(RadixBufs b, RadixState *st, int pass, uint64_t n,
-                                                              int shift, const uint64_t *spl, int n_spl,
-                                                              const uint32_t *hist, uint32_t ntiles,
-                                                              const uint64_t *bases, unsigned int *tickets,
-                                                              unsigned long long *status) {
-  if (!kRange && st->skip[pass]) {
-    if (kOneSweep && blockIdx.x == 0 && threadIdx.x == 0) st->cur[pass + 1] = st->cur[pass];
-    return;
-  }
+// The tile's digit offsets come from the scanned per-tile histograms.
+__global__ void __launch_bounds__(kRxThreads, 2) rx_range_scatter(RadixBufs b, const RadixState *st, uint64_t n,
+                                                                  const uint64_t *spl, int n_spl, const uint32_t *hist,
+                                                                  uint32_t ntiles) {
   extern __shared__ __align__(16) unsigned char rx_smem[];
   RxScatterSmem &sm = *reinterpret_cast<RxScatterSmem *>(rx_smem);
   __shared__ uint64_t s_spl[kRxDigits];
-  __shared__ uint32_t s_tile;
-  const int c = kRange ? 0 : st->cur[pass];
-  const uint64_t *kin = b.keys[c];
-  const uint32_t *vin = b.vals[c];
-  uint64_t *kout = b.keys[1 - c];
-  uint32_t *vout = b.vals[1 - c];
-  if (kOneSweep && threadIdx.x == 0) s_tile = atomicAdd(&tickets[pass], 1u);
+  const uint64_t *kin = b.keys[0];
+  const uint32_t *vin = b.vals[0];
+  uint64_t *kout = b.keys[1];
+  uint32_t *vout = b.vals[1];
   for (int i = threadIdx.x; i < kRxWarps * kRxDigits; i += blockDim.x) (&sm.wcnt[0][0])[i] = 0;
-  if (kRange)
-    for (int i = threadIdx.x; i < n_spl; i += blockDim.x) s_spl[i] = spl[i];
+  for (int i = threadIdx.x; i < n_spl; i += blockDim.x) s_spl[i] = spl[i];
   __syncthreads();
-  const uint32_t tile = kOneSweep ? s_tile : blockIdx.x;
-  if (kOneSweep && tile == 0 && threadIdx.x == 0) st->cur[pass + 1] = 1 - c;  // read by the next pass only
+  const uint32_t tile = blockIdx.x;
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint64_t tbase = (uint64_t)tile * kRxTile;
   const uint64_t wbase = tbase + (uint64_t)w * (32 * kRxItems);
@@ -263,7 +233,7 @@ __global__ void __launch_bounds__(kRxThreads, 2) rx_downsweep(RadixBufs b, Radix
 #pragma unroll
   for (int r = 0; r < kRxItems; ++r) {
     const uint64_t i = wbase + (uint64_t)r * 32 + lane;
-    const uint32_t d = i < n ? key_digit<kRange>(k[r], shift, s_spl, n_spl) : kRxInvalid;
+    const uint32_t d = i < n ? key_range(k[r], s_spl, n_spl) : kRxInvalid;
     const uint32_t peers = __match_any_sync(0xffffffffu, d);
     uint32_t before = 0;
     if (d != kRxInvalid) before = sm.wcnt[w][d];
@@ -282,39 +252,8 @@ __global__ void __launch_bounds__(kRxThreads, 2) rx_downsweep(RadixBufs b, Radix
       sm.wcnt[q][d] = run;
       run += cq;
     }
-    uint64_t before_tile;  // position of the tile's first pair of digit d
-    if (kOneSweep) {
-      volatile unsigned long long *sw = status + (uint64_t)tile * kRxDigits + d;
-      *sw = rx_status_word(tile == 0 ? kRxFlagIncl : kRxFlagAgg, pass, run);
-      uint64_t prefix = 0;  // pairs of digit d in the tiles before this one
-      const uint32_t limit = st->spin_limit;
-      for (uint32_t t = tile; t > 0;) {  // look back over the predecessors' words
-        --t;
-        const volatile unsigned long long *pw = status + (uint64_t)t * kRxDigits + d;
-        uint64_t word = *pw;
-        uint32_t spins = 0;
-        while ((word >> 62) == 0 || (int)((word >> 59) & 7u) != pass) {
-          // give up after the limit, or at once when another tile already gave up
-          if (++spins > limit || ((spins & 1023u) == 0 && *(volatile uint32_t *)&st->err)) {
-            spins = limit + 1;
-            break;
-          }
-          __nanosleep(32);
-          word = *pw;
-        }
-        if (spins > limit) {  // a predecessor never published: report, keep going (a partial
-                              // prefix only lowers this tile's positions, all inside the pass's n)
-          atomicOr(&st->err, 1u);
-          break;
-        }
-        prefix += word & kRxValueMask;
-        if ((word >> 62) == 2) break;
-      }
-      if (tile > 0) *sw = rx_status_word(kRxFlagIncl, pass, prefix + run);
-      before_tile = bases[pass * kRxDigits + d] + prefix;
-    } else {
-      before_tile = st->base[d] + hist[(uint64_t)d * ntiles + tile];
-    }
+    // position of the tile's first pair of digit d
+    const uint64_t before_tile = st->base[d] + hist[(uint64_t)d * ntiles + tile];
     uint32_t x = run;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -349,15 +288,218 @@ __global__ void __launch_bounds__(kRxThreads, 2) rx_downsweep(RadixBufs b, Radix
   }
 }
 
+// One LSD pass: a stable scatter of the pairs by one key byte.  The tile is
+// the block's ticket; its digits' positions come from the one-read histogram
+// (bases) plus a look-back over the status words of the tiles before it.
+//   rank: a warp owns kI * 32 consecutive pairs.  The lanes of a round that
+// share a digit find one another (match_any), their first lane adds them to the
+// warp's counter of the digit and hands the count before them to the others;
+// the rounds' matches and shared-memory atomics are issued back to back, so
+// that the warp waits for one round trip per kB rounds and not for each.
+//   place: keys are regrouped by digit in shared memory while the tiles before
+// publish, then written as runs of consecutive positions; the values follow
+// through the same shared memory.  Holding only one of the two at a time lets
+// 28 warps share an SM, which the latencies here need.
+// Bound by shared-memory wavefronts, barriers and issue rather than by HBM: 24
+// bytes a pair and pass at 3.25 TB/s (0.48 of the measured copy bandwidth, 40M
+// pairs); 1.67 TB/s before, when every round waited for its match_any and its
+// counter, and keys and values together left 16 warps an SM.
+// Lanes of the warp with the same 8-bit digit, from one vote per bit
+// (match_any takes a step per distinct value, about 30 of them for random
+// digits: 0.98 against 0.74 ms for the eight passes over 9.6M random pairs,
+// and 0.70 with the matches found through shared-memory words, which falls to
+// 0.78 on skewed digits where votes take 0.69).
+__device__ __forceinline__ uint32_t same_digit(uint32_t d) {
+  uint32_t peers = 0xffffffffu;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const uint32_t on = (uint32_t)((int32_t)(d << (31 - b)) >> 31);  // all ones where the bit is set
+    peers &= ~(__ballot_sync(0xffffffffu, on != 0) ^ on);
+  }
+  return peers;
+}
+
+template <int kT, int kI, class Off>
+struct RxSweepSmem {
+  uint64_t k[kT * kI];                 // the keys by digit, then the values
+  uint32_t wcnt[kT / 32][kRxDigits];
+  Off off[kRxDigits];  // global position of local position 0 of each digit
+  uint32_t wsum[kRxDigits / 32];
+  uint32_t tile;
+};
+
+template <int kT, int kI, class Off>
+__global__ void __launch_bounds__(kT, 2) rx_sweep(RadixBufs b, RadixState *st, int pass, uint64_t n,
+                                                          const uint64_t *bases, unsigned int *tickets,
+                                                          unsigned long long *status) {
+  constexpr int kTile = kT * kI, kB = 4;
+  static_assert(kT >= kRxDigits && kI % kB == 0 && kTile <= 65536, "a thread per digit, whole batches, 16-bit places");
+  if (st->skip[pass]) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->cur[pass + 1] = st->cur[pass];
+    return;
+  }
+  extern __shared__ __align__(16) unsigned char rx_smem[];
+  RxSweepSmem<kT, kI, Off> &sm = *reinterpret_cast<RxSweepSmem<kT, kI, Off> *>(rx_smem);
+  const int c = st->cur[pass];
+  if (threadIdx.x == 0) sm.tile = atomicAdd(&tickets[pass], 1u);
+  for (int i = threadIdx.x; i < kT / 32 * kRxDigits; i += kT) (&sm.wcnt[0][0])[i] = 0;
+  __syncthreads();
+  const uint32_t tile = sm.tile;
+  if (tile == 0 && threadIdx.x == 0) st->cur[pass + 1] = 1 - c;  // read by the next pass only
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint64_t tbase = (uint64_t)tile * kTile;
+  const uint32_t valid = n - tbase < (uint64_t)kTile ? (uint32_t)(n - tbase) : (uint32_t)kTile;
+  const uint32_t first = w * (32 * kI) + lane;  // the thread's pairs: first + 32 r of the tile
+  const uint64_t *kin = (c ? b.keys[1] : b.keys[0]) + tbase;
+  auto digit = [&](uint64_t k) { return __byte_perm((uint32_t)k, (uint32_t)(k >> 32), pass) & 0xFFu; };
+  // keys past the end are all ones: the last pairs of the tile's last digit
+  uint64_t k[kI];
+#pragma unroll
+  for (int r = 0; r < kI; ++r) k[r] = first + 32 * r < valid ? kin[first + 32 * r] : ~0ull;
+  // rank inside the warp's pairs of the digit, then the place in the tile: two
+  // 16-bit ones per word (registers are what limits the warps here)
+  uint32_t place[kI / 2];
+#pragma unroll
+  for (int r0 = 0; r0 < kI; r0 += kB) {
+    uint32_t peers[kB], before[kB];
+#pragma unroll
+    for (int r = 0; r < kB; ++r) peers[r] = same_digit(digit(k[r0 + r]));
+#pragma unroll
+    for (int r = 0; r < kB; ++r) {
+      before[r] = 0;
+      if ((peers[r] & lanemask_lt()) == 0) before[r] = atomicAdd(&sm.wcnt[w][digit(k[r0 + r])], __popc(peers[r]));
+      __syncwarp();
+    }
+#pragma unroll
+    for (int r = 0; r < kB; ++r) {
+      const uint32_t rank =
+          __shfl_sync(0xffffffffu, before[r], __ffs(peers[r]) - 1) + __popc(peers[r] & lanemask_lt());
+      place[(r0 + r) / 2] = r % 2 ? place[(r0 + r) / 2] | rank << 16 : rank;
+    }
+  }
+  __syncthreads();
+  const uint32_t d = threadIdx.x;
+  uint32_t run = 0, start = 0;  // the tile's pairs of digit d, their first place
+  volatile unsigned long long *sw = status + (uint64_t)tile * kRxDigits + d;
+  uint32_t cnt[kT / 32];
+  if (d < kRxDigits) {
+#pragma unroll
+    for (int q = 0; q < kT / 32; ++q) {
+      cnt[q] = sm.wcnt[q][d];
+      run += cnt[q];
+    }
+    uint32_t x = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= (uint32_t)o) x += y;
+    }
+    if (lane == 31) sm.wsum[w] = x;
+    start = x - run;
+    if (d == kRxDigits - 1) run -= kTile - valid;
+    *sw = rx_status_word(tile == 0 ? kRxFlagIncl : kRxFlagAgg, pass, run);
+  }
+  __syncthreads();
+  if (d < kRxDigits) {  // where each warp's pairs of the digit go
+#pragma unroll
+    for (int q = 0; q < kRxDigits / 32; ++q) start += q < (int)w ? sm.wsum[q] : 0u;
+    uint32_t at = start;
+#pragma unroll
+    for (int q = 0; q < kT / 32; ++q) {
+      sm.wcnt[q][d] = at;
+      at += cnt[q];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kI; ++r) {
+    place[r / 2] += sm.wcnt[w][digit(k[r])] << (r % 2 * 16);
+    sm.k[r % 2 ? place[r / 2] >> 16 : place[r / 2] & 0xFFFFu] = k[r];
+  }
+  const uint32_t *vin = (c ? b.vals[1] : b.vals[0]) + tbase;
+  uint32_t v[kI];
+#pragma unroll
+  for (int r = 0; r < kI; ++r) v[r] = first + 32 * r < valid ? vin[first + 32 * r] : 0u;
+  if (d < kRxDigits) {
+    uint64_t prefix = 0;  // pairs of digit d in the tiles before this one
+    const uint32_t limit = st->spin_limit;
+    bool done = tile == 0;
+    for (uint32_t t = tile; !done;) {  // look back over the predecessors' words, kL of them read at once
+      constexpr uint32_t kL = 4;
+      uint64_t word[kL];
+#pragma unroll
+      for (uint32_t j = 0; j < kL; ++j)
+        word[j] = *(const volatile unsigned long long *)(status + (uint64_t)(t > j ? t - 1 - j : 0) * kRxDigits + d);
+#pragma unroll
+      for (uint32_t j = 0; j < kL; ++j) {
+        if (done) break;
+        uint32_t spins = 0;
+        while ((word[j] >> 62) == 0 || (int)((word[j] >> 59) & 7u) != pass) {
+          // give up after the limit, or at once when another tile already gave up
+          if (++spins > limit || ((spins & 1023u) == 0 && *(volatile uint32_t *)&st->err)) {
+            spins = limit + 1;
+            break;
+          }
+          __nanosleep(32);
+          word[j] = *(const volatile unsigned long long *)(status + (uint64_t)(t - 1 - j) * kRxDigits + d);
+        }
+        if (spins > limit) {  // a predecessor never published: report, keep going (a partial
+                              // prefix only lowers this tile's positions, all inside the pass's n)
+          atomicOr(&st->err, 1u);
+          done = true;
+          break;
+        }
+        prefix += word[j] & kRxValueMask;
+        done = (word[j] >> 62) == 2;  // tile 0's word is always inclusive
+      }
+      t = t > kL ? t - kL : 0;
+      if (t == 0) done = true;
+    }
+    if (tile > 0) *sw = rx_status_word(kRxFlagIncl, pass, prefix + run);
+    sm.off[d] = (Off)(bases[pass * kRxDigits + d] + prefix - start);  // wraps back when added to a position
+  }
+  __syncthreads();
+  uint64_t *kout = c ? b.keys[0] : b.keys[1];
+  uint32_t *vout = c ? b.vals[0] : b.vals[1];
+  uint32_t dg[kI / 4];  // the digits of the places this thread writes
+#pragma unroll
+  for (int j = 0; j < kI; ++j) {
+    const uint32_t t = threadIdx.x + j * kT;
+    const uint64_t key = sm.k[t];
+    const uint32_t g = digit(key);
+    dg[j / 4] = j % 4 ? dg[j / 4] | g << (8 * (j % 4)) : g;
+    if (t < valid) kout[(Off)(sm.off[g] + t)] = key;
+  }
+  __syncthreads();
+  uint32_t *sv = reinterpret_cast<uint32_t *>(sm.k);
+#pragma unroll
+  for (int r = 0; r < kI; ++r) sv[r % 2 ? place[r / 2] >> 16 : place[r / 2] & 0xFFFFu] = v[r];
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kI; ++j) {
+    const uint32_t t = threadIdx.x + j * kT;
+    if (t < valid) vout[(Off)(sm.off[dg[j / 4] >> (8 * (j % 4)) & 0xFFu] + t)] = sv[t];
+  }
+}
+
 constexpr size_t kRxScatterSmem = sizeof(RxScatterSmem);
 
-// the scatter's shared memory is above the 48 KB default: raise the limit once
+// 14 warps a block, two blocks an SM, 72 registers a thread: eight passes over
+// 9.6M / 40M random pairs take 0.666 / 2.36 ms; 512 x 2 (64 registers, spilling
+// more) 0.683 / 2.40, 384 x 3 0.750 / 2.59, 256 x 4 0.723 / 2.48
+constexpr int kSweepThreads = 448, kSweepItems = 16;
+constexpr uint32_t kSweepTile = kSweepThreads * kSweepItems;
+constexpr size_t kRxSweepSmem = sizeof(RxSweepSmem<kSweepThreads, kSweepItems, uint64_t>);
+
+// the scatters' shared memory is above the 48 KB default: raise the limit once
 static vx_status rx_scatter_attr() {
   static bool done = false;
   if (!done) {
-    VX_CUDA_TRY(cudaFuncSetAttribute(rx_downsweep<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kRxScatterSmem));
-    VX_CUDA_TRY(cudaFuncSetAttribute(rx_downsweep<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    VX_CUDA_TRY(cudaFuncSetAttribute(rx_sweep<kSweepThreads, kSweepItems, uint32_t>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRxSweepSmem));
+    VX_CUDA_TRY(cudaFuncSetAttribute(rx_sweep<kSweepThreads, kSweepItems, uint64_t>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRxSweepSmem));
+    VX_CUDA_TRY(cudaFuncSetAttribute(rx_range_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kRxScatterSmem));
     done = true;
   }
@@ -571,28 +713,27 @@ static vx_status radix_result(char *temp, cudaStream_t s, int *cur) {
 // buffer st->cur[npass] (0 or 1).
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass,
                              uint32_t spin_limit) {
-  uint32_t nt = ntiles_of(n);
+  const uint32_t nt = (uint32_t)((n + kSweepTile - 1) / kSweepTile);
   RadixState *st = radix_state_of(temp);
   unsigned long long *bh = (unsigned long long *)(temp + kStateBytes);
-  uint32_t *hist = (uint32_t *)(temp + kStateBytes + kByteHistBytes);
-  VX_CUDA_TRY(cudaMemsetAsync(bh, 0, kByteHistBytes, s));
+  uint64_t *bases = (uint64_t *)(temp + kStateBytes + kByteHistBytes);
+  unsigned int *tickets = (unsigned int *)((char *)bases + kBasesBytes);
+  unsigned long long *status = (unsigned long long *)((char *)tickets + kTicketBytes);
   if (n == 0) {
-    VX_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(RadixState), s));
+    VX_CUDA_TRY(cudaMemsetAsync(temp, 0, kStateBytes + kByteHistBytes, s));
     return VX_OK;
   }
   VX_TRY(rx_scatter_attr());
-  uint64_t *bases = (uint64_t *)hist;
-  unsigned int *tickets = (unsigned int *)((char *)hist + kBasesBytes);
-  unsigned long long *status = (unsigned long long *)((char *)hist + kBasesBytes + kTicketBytes);
-  // tickets and status words: cleared once, the words carry their pass number
-  VX_CUDA_TRY(cudaMemsetAsync(tickets, 0, kTicketBytes + (uint64_t)kRxDigits * nt * 8, s));
-  int g = (int)std::min<uint64_t>((n + kRxThreads - 1) / kRxThreads, (uint64_t)num_sms * 4);
-  rx_byte_hist<<<g, kRxThreads, 0, s>>>(b, n, bh);
-  rx_init_state<<<1, 32, 0, s>>>(st, bh, n, spin_limit ? spin_limit : kRxSpinLimit);
-  rx_init_bases<<<8, kRxDigits, 0, s>>>(bh, bases);
+  // histograms, tickets and status words (the words carry their pass number)
+  VX_CUDA_TRY(cudaMemsetAsync(bh, 0, kByteHistBytes + kBasesBytes + kTicketBytes + (uint64_t)kRxDigits * nt * 8, s));
+  const int g = (int)std::min<uint64_t>((n + kRxThreads - 1) / kRxThreads, (uint64_t)num_sms * 6);
+  auto hist = npass == 1 ? rx_byte_hist<1> : npass == 2 ? rx_byte_hist<2> : npass == 3 ? rx_byte_hist<3> : rx_byte_hist<8>;
+  hist<<<g, kRxThreads, 0, s>>>(b.keys[0], n, bh);
+  rx_init<<<npass, kRxDigits, 0, s>>>(st, bh, bases, n, spin_limit ? spin_limit : kRxSpinLimit);
+  // positions take 32 bits below 2^32 pairs
+  auto sweep = n >> 32 ? rx_sweep<kSweepThreads, kSweepItems, uint64_t> : rx_sweep<kSweepThreads, kSweepItems, uint32_t>;
   for (int pass = 0; pass < npass; ++pass)  // a skipped pass returns at once and keeps the buffer
-    rx_downsweep<false, true><<<nt, kRxThreads, kRxScatterSmem, s>>>(b, st, pass, n, 8 * pass, nullptr, 0, nullptr, nt,
-                                                                      bases, tickets, status);
+    sweep<<<nt, kSweepThreads, kRxSweepSmem, s>>>(b, st, pass, n, bases, tickets, status);
   VX_CUDA_TRY(cudaGetLastError());
   return VX_OK;
 }
@@ -608,13 +749,11 @@ vx_status range_partition_enqueue(RadixBufs b, uint64_t n, const uint64_t *spl, 
   VX_TRY(rx_scatter_attr());
   VX_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(RadixState), s));
   if (n) {
-    rx_upsweep<true><<<nt, kRxThreads, 0, s>>>(b, st, 0, n, 0, spl, (int)P - 1, hist, nt);
-    rx_scan_rows<<<kRxDigits, 1024, 0, s>>>(hist, nt, st, 0, false);
+    rx_upsweep<<<nt, kRxThreads, 0, s>>>(b.keys[0], n, spl, (int)P - 1, hist, nt);
+    rx_scan_rows<<<kRxDigits, 1024, 0, s>>>(hist, nt, st);
   }
-  rx_scan_totals<<<1, kRxDigits, 0, s>>>(st, 0, n, false);
-  if (n)
-    rx_downsweep<true, false><<<nt, kRxThreads, kRxScatterSmem, s>>>(b, st, 0, n, 0, spl, (int)P - 1, hist, nt,
-                                                                      nullptr, nullptr, nullptr);
+  rx_scan_totals<<<1, kRxDigits, 0, s>>>(st, n);
+  if (n) rx_range_scatter<<<nt, kRxThreads, kRxScatterSmem, s>>>(b, st, n, spl, (int)P - 1, hist, nt);
   VX_CUDA_TRY(cudaGetLastError());
   return VX_OK;
 }
@@ -1166,7 +1305,7 @@ vx_status sort_contiguous(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
     VX_TRY(run_pipeline(ctx, sp, &es));
     ss.bytes_h2d += es.bytes_h2d;
     ss.bytes_d2h += es.bytes_d2h;
-    ss.kernel_launches += es.kernel_launches * 35;  // byte histogram, state, 8 x 4 passes, publish
+    ss.kernel_launches += es.kernel_launches * 11;  // byte histogram, state, 8 passes, publish
     ss.ms_sort_kernel += es.ms_kernel;
     ss.radix_pass_pairs += sp.pass_pairs;
   }
