@@ -440,7 +440,10 @@ typedef struct {
  * (opts->runs_mode).
  * Both plans and any splitters give the same output; they decide only where
  * to cut.  The intermediate is opts->host_scratch when it holds 12 n bytes,
- * else allocated for the call. */
+ * else allocated for the call.  With the PARTITION plan and neither
+ * max_slot_pairs nor region_slack_pct given, an input that fits the arena
+ * beside the passes' slots (about 13 bytes a pair) keeps its partitions there
+ * and uses no intermediate. */
 vx_status vx_sort(vx_ctx *ctx, int32_t key_col, int32_t rowid_col, uint64_t *out_keys, uint32_t *out_rowids,
                   const vx_sort_opts *opts, vx_sort_stats *stats);
 

@@ -122,6 +122,30 @@ __global__ void __launch_bounds__(kRxDigits) rx_scan_totals(RadixState *st, uint
   if (d == 0) st->base[kRxDigits] = n;
 }
 
+// Resident partitions: where each partition's region of the arena starts, how
+// many pairs it takes and how many it holds.
+struct RxRegions {
+  uint64_t off[kRxDigits], cap[kRxDigits], used[kRxDigits];
+  uint64_t dest[kRxDigits];  // of the chunk in work: position of the partition's first pair
+  uint32_t full;             // a region was too small: nothing is scattered any more
+};
+
+// one block of 256 threads: the chunk's partitions go behind what their
+// regions hold
+__global__ void __launch_bounds__(kRxDigits) rx_place(const RadixState *st, RxRegions *rg, uint32_t P) {
+  const uint32_t d = threadIdx.x;
+  const uint64_t t = d < P ? st->totals[d] : 0, u = d < P ? rg->used[d] : 0;
+  const int over = __syncthreads_or(d < P && t > rg->cap[d] - u);
+  if (over) {
+    if (d == 0) rg->full = 1;
+    return;
+  }
+  if (d < P) {
+    rg->dest[d] = rg->off[d] + u;
+    rg->used[d] = u + t;
+  }
+}
+
 // histograms of the low npass key bytes in one read (constant digits are
 // skipped later)
 template <int kP>
@@ -204,10 +228,12 @@ __device__ __forceinline__ uint64_t rx_status_word(uint64_t flag, int pass, uint
 // 16 rounds of 32 consecutive pairs), regroup the tile by digit in shared
 // memory, then write each digit's run with consecutive threads on consecutive
 // output positions, so stores leave the SM as contiguous runs.
-// The tile's digit offsets come from the scanned per-tile histograms.
+// The tile's digit offsets come from the scanned per-tile histograms, behind
+// the partitions' starts in the chunk (rg null) or in their regions.
 __global__ void __launch_bounds__(kRxThreads, 2) rx_range_scatter(RadixBufs b, const RadixState *st, uint64_t n,
                                                                   const uint64_t *spl, int n_spl, const uint32_t *hist,
-                                                                  uint32_t ntiles) {
+                                                                  uint32_t ntiles, const RxRegions *rg) {
+  if (rg && rg->full) return;
   extern __shared__ __align__(16) unsigned char rx_smem[];
   RxScatterSmem &sm = *reinterpret_cast<RxScatterSmem *>(rx_smem);
   __shared__ uint64_t s_spl[kRxDigits];
@@ -253,7 +279,8 @@ __global__ void __launch_bounds__(kRxThreads, 2) rx_range_scatter(RadixBufs b, c
       run += cq;
     }
     // position of the tile's first pair of digit d
-    const uint64_t before_tile = st->base[d] + hist[(uint64_t)d * ntiles + tile];
+    const uint64_t before_tile =
+        d <= n_spl ? (rg ? rg->dest[d] : st->base[d]) + hist[(uint64_t)d * ntiles + tile] : 0;
     uint32_t x = run;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -753,7 +780,23 @@ vx_status range_partition_enqueue(RadixBufs b, uint64_t n, const uint64_t *spl, 
     rx_scan_rows<<<kRxDigits, 1024, 0, s>>>(hist, nt, st);
   }
   rx_scan_totals<<<1, kRxDigits, 0, s>>>(st, n);
-  if (n) rx_range_scatter<<<nt, kRxThreads, kRxScatterSmem, s>>>(b, st, n, spl, (int)P - 1, hist, nt);
+  if (n) rx_range_scatter<<<nt, kRxThreads, kRxScatterSmem, s>>>(b, st, n, spl, (int)P - 1, hist, nt, nullptr);
+  VX_CUDA_TRY(cudaGetLastError());
+  return VX_OK;
+}
+
+// The same scatter of n > 0 pairs into the partitions' regions of b.keys[1] /
+// b.vals[1], each behind what the region holds.
+static vx_status region_partition_enqueue(RadixBufs b, uint64_t n, const uint64_t *spl, uint32_t P, RxRegions *rg,
+                                          char *temp, cudaStream_t s) {
+  const uint32_t nt = ntiles_of(n);
+  RadixState *st = radix_state_of(temp);
+  uint32_t *hist = (uint32_t *)(temp + kStateBytes + kByteHistBytes);
+  VX_TRY(rx_scatter_attr());
+  rx_upsweep<<<nt, kRxThreads, 0, s>>>(b.keys[0], n, spl, (int)P - 1, hist, nt);
+  rx_scan_rows<<<kRxDigits, 1024, 0, s>>>(hist, nt, st);
+  rx_place<<<1, kRxDigits, 0, s>>>(st, rg, P);
+  rx_range_scatter<<<nt, kRxThreads, kRxScatterSmem, s>>>(b, st, n, spl, (int)P - 1, hist, nt, rg);
   VX_CUDA_TRY(cudaGetLastError());
   return VX_OK;
 }
@@ -1064,11 +1107,243 @@ struct SortPass : ExKernel {
   }
 };
 
+// ---- partitions that stay in the arena
+// When the arena holds all pairs beside the slots of both passes, pass 1
+// scatters the chunks straight into the partitions' regions and pass 2 sorts
+// each partition where it is (the other buffer in a slot) and stores it: the
+// pairs cross the link once in each direction instead of twice.  67M uniform
+// pairs (805 MB) under 1 GiB: 10.3 ms, 13.7 through host memory; 300M (3.6 GB)
+// under 4.5 GiB: 39 ms, about 62.  Bound by the link one way, then the other,
+// and by the partition sorts (5.0 of the 5.7 ms of pass 2).
+struct ResidentPlan {
+  std::vector<uint64_t> off, cap;  // regions, pairs
+  uint64_t pairs = 0;              // all regions
+  uint64_t R = 0, jcap = 0;        // pairs per slot of pass 1 and pass 2
+  int S1 = 0, S2 = 0;
+};
+
+struct ResidentPartitionPass : ExKernel {
+  const uint64_t *keys;
+  const uint32_t *vals;
+  uint64_t n, R;
+  int S;
+  uint32_t P;
+  const uint64_t *d_spl;
+  uint64_t *res_keys;
+  uint32_t *res_vals;
+  RxRegions *rg;
+  uint64_t size() override { return (n + R - 1) / R; }
+  int n_slots() override { return S; }
+  uint64_t rows(uint64_t it) const { return std::min(R, n - it * R); }
+  uint64_t kb() const { return (8 * R + 255) & ~255ull; }
+  uint64_t vb() const { return (4 * R + 255) & ~255ull; }
+  static uint64_t bytes(uint64_t R) { return (8 * R + 255) / 256 * 256 + (4 * R + 255) / 256 * 256 + radix_temp_bytes(R); }
+  uint64_t slot_bytes() override { return bytes(R); }
+  void inputs(uint64_t it, char *slot, std::vector<CopyOp> &h2d) override {
+    h2d.push_back({keys + it * R, slot, 8 * rows(it)});
+    h2d.push_back({vals + it * R, slot + kb(), 4 * rows(it)});
+  }
+  vx_status kernel(char *slot, uint64_t it, cudaStream_t s) override {
+    RadixBufs b;
+    b.keys[0] = (uint64_t *)slot;
+    b.vals[0] = (uint32_t *)(slot + kb());
+    b.keys[1] = res_keys;
+    b.vals[1] = res_vals;
+    return region_partition_enqueue(b, rows(it), d_spl, P, rg, slot + kb() + vb(), s);
+  }
+};
+
+struct ResidentSortPass : ExKernel {
+  vx_ctx *ctx;
+  uint64_t cap;
+  struct Job {
+    uint64_t *k;
+    uint32_t *v;
+    uint64_t n, at;  // pairs, output position
+    bool sorted;     // one key value: already in input order
+  };
+  std::vector<Job> jobs;
+  uint64_t *out_keys;
+  uint32_t *out_vals;
+  int S;
+  uint64_t pass_pairs = 0;
+  uint64_t size() override { return jobs.size(); }
+  int n_slots() override { return S; }
+  int max_in_flight() override { return S; }
+  uint64_t kb() const { return (8 * cap + 255) & ~255ull; }
+  uint64_t vb() const { return (4 * cap + 255) & ~255ull; }
+  uint64_t slot_bytes() override { return ResidentPartitionPass::bytes(cap); }
+  void inputs(uint64_t, char *, std::vector<CopyOp> &) override {}
+  RadixBufs bufs(const Job &j, char *slot) const {
+    RadixBufs b;
+    b.keys[0] = j.k;
+    b.vals[0] = j.v;
+    b.keys[1] = (uint64_t *)slot;
+    b.vals[1] = (uint32_t *)(slot + kb());
+    return b;
+  }
+  vx_status kernel(char *slot, uint64_t it, cudaStream_t s) override {
+    const Job &j = jobs[it];
+    if (j.sorted) return VX_OK;
+    char *temp = slot + kb() + vb();
+    VX_TRY(radix_sort_enqueue(bufs(j, slot), j.n, temp, s, ctx->num_sms, 8, ctx->cfg.lookback_spin_limit));
+    return radix_publish_enqueue(temp, ctx->d_scalars + 64 + (it % S), s);
+  }
+  bool has_outputs() override { return true; }
+  vx_status outputs(uint64_t it, char *slot, std::vector<CopyOp> &d2h) override {
+    const Job &j = jobs[it];
+    int c = 0;
+    if (!j.sorted) {
+      const uint64_t word = ((volatile uint64_t *)ctx->h_scalars)[64 + (it % S)];
+      if (word >> 16 & 1) {
+        set_error("radix sort of partition job %llu: a look-back wait gave up", (unsigned long long)it);
+        return VX_E_TIMEOUT;
+      }
+      c = (int)(word & 0xFF);
+      pass_pairs += j.n * ((word >> 8) & 0xFF);
+    }
+    const RadixBufs b = bufs(j, slot);
+    d2h.push_back({b.keys[c], out_keys + j.at, 8 * j.n});
+    d2h.push_back({b.vals[c], out_vals + j.at, 4 * j.n});
+    return VX_OK;
+  }
+};
+
+// partition p of spl's P = spl.size() + 1 holds one key value
+bool single_key_partition(const std::vector<uint64_t> &spl, uint32_t p) {
+  const uint64_t lo = p == 0 ? 0 : spl[p - 1];
+  return p < spl.size() ? (spl[p] > lo && spl[p] - lo == 1) : lo == UINT64_MAX;
+}
+
+// Partitions requested so that the regions, and two slots of pass 2 beside
+// them, fit `avail` bytes with room for uneven partitions; 0: they do not fit.
+uint32_t resident_partitions(uint64_t n, uint64_t avail, double headroom) {
+  const double left = (double)avail - 12.0 * 1.03 * (double)n - (1 << 20);
+  if (left <= 0) return 0;
+  const double jcap = left / (2 * 12.6);
+  // at most 12M pairs a job, so that the stores start early
+  const double P = std::max(std::ceil(headroom * (double)n / jcap), std::ceil((double)n / 12e6));
+  return P > 64 ? 0u : std::max<uint32_t>((uint32_t)P, 4);
+}
+
+// Regions from the sample's count in each partition: the estimate plus 0.2 %
+// and six standard deviations (a region that is too small all the same ends the
+// attempt).  False if regions and slots do not fit `avail` bytes.
+bool resident_layout(uint64_t n, uint64_t m, const std::vector<uint64_t> &spl, const std::vector<uint64_t> &srank,
+                     uint64_t avail, int S, ResidentPlan *rp) {
+  const uint32_t P = (uint32_t)spl.size() + 1;
+  rp->off.resize(P);
+  rp->cap.resize(P);
+  rp->pairs = rp->jcap = 0;
+  const double scale = (double)n / (double)m;
+  for (uint32_t p = 0; p < P; ++p) {
+    const double cnt = (double)((p + 1 < P ? srank[p] : m) - (p ? srank[p - 1] : 0));
+    const double est = 1.002 * cnt * scale + 6.0 * std::sqrt(cnt + 1.0) * scale + kRxTile;
+    rp->cap[p] = (std::min<uint64_t>(n, (uint64_t)std::ceil(est)) + 127) / 128 * 128;
+    rp->off[p] = rp->pairs;
+    rp->pairs += rp->cap[p];
+    if (!single_key_partition(spl, p)) rp->jcap = std::max(rp->jcap, rp->cap[p]);
+  }
+  rp->jcap = std::max<uint64_t>(rp->jcap, kRxTile);
+  const uint64_t fixed = 12 * rp->pairs + sizeof(RxRegions) + 4096;
+  if (fixed >= avail) return false;
+  const uint64_t left = avail - fixed;
+  rp->S2 = (int)std::min<uint64_t>(kMaxSortSlots, left / (ResidentPartitionPass::bytes(rp->jcap) + 256));
+  if (rp->S2 < 2) return false;
+  rp->S1 = S;
+  for (rp->R = std::min<uint64_t>(std::max<uint64_t>(n / 16, 1 << 20), kPipelineRows) / kRxTile * kRxTile;
+       rp->R >= (1 << 18); rp->R = rp->R / 2 / kRxTile * kRxTile)
+    if ((uint64_t)S * (ResidentPartitionPass::bytes(rp->R) + 256) <= left) return true;
+  return false;
+}
+
+// Both passes with resident partitions.  *done = false: a region was too small
+// (nothing has been written to the output; the caller sorts the other way).
+vx_status resident_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals, uint64_t n, uint64_t *out_keys,
+                        uint32_t *out_vals, const uint64_t *d_spl, const std::vector<uint64_t> &spl,
+                        const ResidentPlan &rp, vx_sort_stats &ss, bool *done) {
+  const uint32_t P = (uint32_t)spl.size() + 1;
+  *done = false;
+  DevBuf mem;
+  mem.arena = &ctx->arena;
+  const uint64_t kb = (8 * rp.pairs + 255) & ~255ull, vb = (4 * rp.pairs + 255) & ~255ull;
+  mem.p = ctx->arena.alloc(kb + vb + sizeof(RxRegions));
+  if (!mem.p) return VX_OK;
+  uint64_t *res_keys = mem.as<uint64_t>();
+  uint32_t *res_vals = (uint32_t *)(mem.as<char>() + kb);
+  RxRegions *rg = (RxRegions *)(mem.as<char>() + kb + vb);
+  cudaStream_t s = ctx->s_compute;
+  double t0 = now_ms();
+  auto h = std::make_unique<RxRegions>();
+  memset(h.get(), 0, sizeof(RxRegions));
+  for (uint32_t p = 0; p < P; ++p) {
+    h->off[p] = rp.off[p];
+    h->cap[p] = rp.cap[p];
+  }
+  VX_CUDA_TRY(cudaMemcpyAsync(rg, h.get(), sizeof(RxRegions), cudaMemcpyHostToDevice, s));
+  {
+    ResidentPartitionPass pp;
+    pp.keys = keys;
+    pp.vals = vals;
+    pp.n = n;
+    pp.R = rp.R;
+    pp.S = rp.S1;
+    pp.P = P;
+    pp.d_spl = d_spl;
+    pp.res_keys = res_keys;
+    pp.res_vals = res_vals;
+    pp.rg = rg;
+    ExecStats es;
+    VX_TRY(run_pipeline(ctx, pp, &es));
+    VX_CUDA_TRY(cudaMemcpyAsync(h.get(), rg, sizeof(RxRegions), cudaMemcpyDeviceToHost, s));
+    VX_CUDA_TRY(cudaStreamSynchronize(s));
+    ss.bytes_h2d += es.bytes_h2d;
+    ss.kernel_launches += es.kernel_launches * 4;  // upsweep, row scan, placement, scatter
+  }
+  ss.ms_partition += now_ms() - t0;
+  if (h->full) return VX_OK;
+  t0 = now_ms();
+  ResidentSortPass sp;
+  sp.ctx = ctx;
+  sp.cap = rp.jcap;
+  sp.out_keys = out_keys;
+  sp.out_vals = out_vals;
+  sp.S = rp.S2;
+  uint64_t at = 0, mx = 0, mn = UINT64_MAX;
+  for (uint32_t p = 0; p < P; ++p) {
+    const uint64_t c = h->used[p];
+    mx = std::max(mx, c);
+    mn = std::min(mn, c);
+    const bool one = single_key_partition(spl, p);
+    if (c) {
+      ss.passthrough_partitions += one;
+      sp.jobs.push_back({res_keys + rp.off[p], res_vals + rp.off[p], c, at, one});
+    }
+    at += c;
+  }
+  ExecStats es;
+  VX_TRY(run_pipeline(ctx, sp, &es));
+  ss.bytes_h2d += es.bytes_h2d;
+  ss.bytes_d2h += es.bytes_d2h;
+  ss.kernel_launches += es.kernel_launches * 11;  // byte histogram, state, 8 passes, publish
+  ss.ms_sort_kernel += es.ms_kernel;
+  ss.radix_pass_pairs += sp.pass_pairs;
+  ss.ms_sort += now_ms() - t0;
+  ss.n_partitions = P;
+  ss.max_partition = mx;
+  ss.min_partition = mn;
+  ss.imbalance = (double)mx / ((double)n / P);
+  ss.contiguous_layout = 1;
+  *done = true;
+  return VX_OK;
+}
+
 }  // namespace
 
 // sorts contiguous host pairs (keys/vals mapped or pinned) into out
-vx_status sort_contiguous(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals, const uint64_t *dev_keys, uint64_t n,
-                          uint64_t *out_keys, uint32_t *out_vals, const vx_sort_opts &o, vx_sort_stats &ss, int depth) {
+static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals, const uint64_t *dev_keys,
+                            uint64_t n, uint64_t *out_keys, uint32_t *out_vals, const vx_sort_opts &o,
+                            vx_sort_stats &ss, int depth, bool may_reside) {
   const int S = std::max(2, ctx->cfg.n_slots);
   const uint64_t avail = ctx->arena.largest_free();
   // pairs per slot: (2 x 12 B + histograms) per pair, S slots
@@ -1133,28 +1408,60 @@ vx_status sort_contiguous(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
     return VX_E_NOMEM;
   }
   uint64_t *d_spl = splbuf.as<uint64_t>();
+  const uint64_t pass_avail = ctx->arena.largest_free();  // for the passes, once the sample is gone
   VX_TRY(sample_and_sort(ctx, dev_keys, n, m, o.seed + (uint64_t)depth * 7919, sbuf, &sorted));
   double ms_train = 0;
   uint32_t n_spl = 0;
-  VX_TRY(splitters_from_sample(ctx, o.partitioner, sorted, m, P, d_spl, o.mlp_steps, &ms_train, &n_spl));
-  P = n_spl + 1;  // partitions after heavy-key isolation
-  std::vector<uint64_t> spl(n_spl), srank(n_spl);
-  if (n_spl) {
-    DevBuf rbuf;
-    rbuf.arena = &ctx->arena;
-    rbuf.p = ctx->arena.alloc(8 * n_spl);
-    if (!rbuf.p) return VX_E_NOMEM;
-    sample_ranks_kernel<<<1, 128, 0, ctx->s_compute>>>(sorted, m, d_spl, n_spl, rbuf.as<uint64_t>());
-    VX_CUDA_TRY(cudaGetLastError());
-    VX_CUDA_TRY(cudaMemcpyAsync(spl.data(), d_spl, 8 * n_spl, cudaMemcpyDeviceToHost, ctx->s_compute));
-    VX_CUDA_TRY(cudaMemcpyAsync(srank.data(), rbuf.p, 8 * n_spl, cudaMemcpyDeviceToHost, ctx->s_compute));
+  std::vector<uint64_t> spl, srank;
+  // splitters for `want` requested partitions and the sample's rank of each
+  auto cut = [&](uint32_t want) -> vx_status {
+    double ms = 0;
+    VX_TRY(splitters_from_sample(ctx, o.partitioner, sorted, m, want, d_spl, o.mlp_steps, &ms, &n_spl));
+    ms_train += ms;
+    P = n_spl + 1;  // partitions after heavy-key isolation
+    spl.resize(n_spl);
+    srank.resize(n_spl);
+    if (n_spl) {
+      DevBuf rbuf;
+      rbuf.arena = &ctx->arena;
+      rbuf.p = ctx->arena.alloc(8 * n_spl);
+      if (!rbuf.p) return VX_E_NOMEM;
+      sample_ranks_kernel<<<1, 128, 0, ctx->s_compute>>>(sorted, m, d_spl, n_spl, rbuf.as<uint64_t>());
+      VX_CUDA_TRY(cudaGetLastError());
+      VX_CUDA_TRY(cudaMemcpyAsync(spl.data(), d_spl, 8 * n_spl, cudaMemcpyDeviceToHost, ctx->s_compute));
+      VX_CUDA_TRY(cudaMemcpyAsync(srank.data(), rbuf.p, 8 * n_spl, cudaMemcpyDeviceToHost, ctx->s_compute));
+    }
     VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
+    return VX_OK;
+  };
+  // resident partitions, where the caller has not bounded the slots or the
+  // regions: a smooth model's partitions are less even than the sample's
+  const uint32_t P_out = P;
+  ResidentPlan rp;
+  bool reside = false;
+  if (may_reside && depth == 0 && !o.max_slot_pairs && !o.region_slack_pct) {
+    uint32_t P_in = resident_partitions(n, pass_avail, o.partitioner == VX_PART_LEARNED_MLP ? 1.4 : 1.2);
+    if (P_in && o.n_partitions > 1) P_in = (uint32_t)o.n_partitions;
+    if (P_in) {
+      VX_TRY(cut(P_in));
+      reside = resident_layout(n, m, spl, srank, pass_avail, S, &rp);
+    }
+    if (!reside && P_in != P_out) n_spl = 0, spl.clear(), P_in = 0;
+    if (!P_in) VX_TRY(cut(P_out));
+  } else {
+    VX_TRY(cut(P_out));
   }
-  VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
   sbuf.release();
   ss.ms_sample += now_ms() - ts - ms_train;
   ss.ms_train += ms_train;
   if (depth == 0 && o.splitters_out) memcpy(o.splitters_out, spl.data(), 8 * n_spl);
+  if (reside) {
+    bool done = false;
+    VX_TRY(resident_sort(ctx, keys, vals, n, out_keys, out_vals, d_spl, spl, rp, ss, &done));
+    if (done) return VX_OK;
+    splbuf.release();
+    return sort_pairs(ctx, keys, vals, dev_keys, n, out_keys, out_vals, o, ss, depth, false);
+  }
 
   // partition-pass chunks of kPipelineRows pairs: long enough for efficient
   // copies (576 MB), short enough that the pass pipelines over many chunks
@@ -1310,10 +1617,8 @@ vx_status sort_contiguous(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
     ss.radix_pass_pairs += sp.pass_pairs;
   }
   for (uint32_t p : big) {
-    const uint64_t lo = p == 0 ? 0 : spl[p - 1];
-    const bool single_key = p + 1 < P ? (spl[p] > lo && spl[p] - lo == 1) : lo == UINT64_MAX;
     std::vector<Extent> ex = extents(p);
-    if (single_key) {  // already in input order: copy through
+    if (single_key_partition(spl, p)) {  // already in input order: copy through
       uint64_t at = poff[p];
       for (const Extent &e : ex) {
         parallel_copy(out_keys + at, e.k, 8 * e.len);
@@ -1345,11 +1650,16 @@ vx_status sort_contiguous(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
     VX_CUDA_TRY(cudaHostGetDevicePointer(&dk, tk, 0));
     vx_sort_opts o2 = o;
     o2.n_partitions = 0;
-    VX_TRY(sort_contiguous(ctx, tk, tv, (const uint64_t *)dk, psize[p], out_keys + poff[p], out_vals + poff[p], o2,
-                           ss, depth + 1));
+    VX_TRY(sort_pairs(ctx, tk, tv, (const uint64_t *)dk, psize[p], out_keys + poff[p], out_vals + poff[p], o2, ss,
+                      depth + 1, false));
   }
   ss.ms_sort += now_ms() - tq;
   return VX_OK;
+}
+
+vx_status sort_contiguous(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals, const uint64_t *dev_keys, uint64_t n,
+                          uint64_t *out_keys, uint32_t *out_vals, const vx_sort_opts &o, vx_sort_stats &ss, int depth) {
+  return sort_pairs(ctx, keys, vals, dev_keys, n, out_keys, out_vals, o, ss, depth, true);
 }
 
 }  // namespace vx
