@@ -443,7 +443,8 @@ typedef struct {
  * else allocated for the call.  With the PARTITION plan and neither
  * max_slot_pairs nor region_slack_pct given, an input that fits the arena
  * beside the passes' slots (about 13 bytes a pair) keeps its partitions there
- * and uses no intermediate. */
+ * and uses no intermediate; so does the MERGE plan without max_slot_pairs
+ * (about 15 bytes a pair, more when the partitions are few). */
 vx_status vx_sort(vx_ctx *ctx, int32_t key_col, int32_t rowid_col, uint64_t *out_keys, uint32_t *out_rowids,
                   const vx_sort_opts *opts, vx_sort_stats *stats);
 

@@ -160,7 +160,8 @@ struct MergeRound {
   uint32_t *vout;
   uint64_t n;
   uint32_t nseg;
-  uint64_t seg[kMaxRuns + 1];  // segment s = [seg[s], seg[s + 1]) of the input buffer
+  uint64_t seg[kMaxRuns + 1];  // segment s has seg[s + 1] - seg[s] pairs; pair q's outputs start at seg[2q]
+  uint64_t src[kMaxRuns];      // and starts at src[s] of the input
 };
 
 // elements of a among the first d outputs of the stable merge of a and b
@@ -174,9 +175,9 @@ __device__ __forceinline__ I merge_path(const uint64_t *a, I na, const uint64_t 
   return lo;
 }
 
-// pair of segments holding output position t, and its bounds
+// pair of segments holding output position t: its outputs and its two inputs
 struct PairAt {
-  uint64_t base, amid, pend;
+  uint64_t base, pend, na, nb, a, b;
 };
 __device__ __forceinline__ PairAt pair_at(const MergeRound &p, uint64_t t) {
   const uint32_t npairs = (p.nseg + 1) / 2;
@@ -185,7 +186,15 @@ __device__ __forceinline__ PairAt pair_at(const MergeRound &p, uint64_t t) {
     const uint32_t mid = (qlo + qhi + 1) / 2;
     if (p.seg[2 * mid] <= t) qlo = mid; else qhi = mid - 1;
   }
-  return PairAt{p.seg[2 * qlo], p.seg[2 * qlo + 1], p.seg[2 * qlo + 2 < p.nseg ? 2 * qlo + 2 : p.nseg]};
+  const uint32_t s0 = 2 * qlo, s1 = s0 + 1;
+  PairAt r;
+  r.base = p.seg[s0];
+  r.na = p.seg[s1] - r.base;
+  r.a = p.src[s0];
+  r.nb = s1 < p.nseg ? p.seg[s1 + 1] - p.seg[s1] : 0;  // an odd last segment is copied
+  r.b = s1 < p.nseg ? p.src[s1] : 0;
+  r.pend = r.base + r.na + r.nb;
+  return r;
 }
 
 // Merge-path cuts of a round, one thread per tile boundary: cut[b] = the
@@ -201,7 +210,7 @@ __global__ void merge_cuts_kernel(const MergeRound p, uint64_t *cut, uint64_t n_
       continue;
     }
     const PairAt q = pair_at(p, t);
-    cut[b] = merge_path<uint64_t>(p.kin + q.base, q.amid - q.base, p.kin + q.amid, q.pend - q.amid, t - q.base);
+    cut[b] = merge_path<uint64_t>(p.kin + q.a, q.na, p.kin + q.b, q.nb, t - q.base);
   }
 }
 
@@ -212,10 +221,10 @@ __global__ void __launch_bounds__(kMergeThreads) merge_round_kernel(const MergeR
   const uint64_t t_end = t0 + kMergeTile < p.n ? t0 + kMergeTile : p.n;
   while (t0 < t_end) {  // the outputs of one pair at a time (a tile may span pairs)
     const PairAt q = pair_at(p, t0);
-    const uint64_t base = q.base, amid = q.amid, pend = q.pend;
+    const uint64_t base = q.base, pend = q.pend, na = q.na;
     const uint64_t t1 = t_end < pend ? t_end : pend;
-    const uint64_t *A = p.kin + base, *B = p.kin + amid;
-    const uint64_t na = amid - base, nb = pend - amid;
+    const uint64_t *A = p.kin + q.a, *B = p.kin + q.b;
+    const uint32_t *VA = p.vin + q.a, *VB = p.vin + q.b;
     const uint64_t d0 = t0 - base, d1 = t1 - base;
     // cuts at the tile's own boundaries come precomputed; a pair boundary
     // inside the tile is where a pair starts (cut 0) or ends (cut na)
@@ -226,10 +235,10 @@ __global__ void __launch_bounds__(kMergeThreads) merge_round_kernel(const MergeR
     for (uint32_t x = threadIdx.x; x < L; x += kMergeThreads) {
       if (x < la) {
         sk[x] = A[i0 + x];
-        sv[x] = p.vin[base + i0 + x];
+        sv[x] = VA[i0 + x];
       } else {
         sk[x] = B[j0 + x - la];
-        sv[x] = p.vin[amid + j0 + x - la];
+        sv[x] = VB[j0 + x - la];
       }
     }
     __syncthreads();
@@ -265,31 +274,36 @@ __global__ void __launch_bounds__(kMergeThreads) merge_round_kernel(const MergeR
   }
 }
 
-// Enqueues the merge of the nseg segments seg[0..nseg] of b.keys[0]/b.vals[0]
-// (n pairs) on s; returns the buffer that holds the result and adds the
-// executed rounds to *rounds.
+// Enqueues the merge of segments of kin/vin (segment s starts at src[s] and
+// has seg[s + 1] - seg[s] pairs, n in all) on s: the first round writes buffer
+// `first` of b, the next ones alternate (kin/vin may be the other buffer).
+// Returns the buffer that holds the result, or -1 for a single segment (nothing
+// is written); adds the executed rounds to *rounds.
 // cuts: device scratch of n / kMergeTile + 2 words
-int merge_enqueue(RadixBufs b, uint64_t n, const std::vector<uint64_t> &seg, uint64_t *cuts, cudaStream_t s,
-                  uint64_t *rounds) {
-  int c = 0;
-  std::vector<uint64_t> cur = seg;
+int merge_enqueue(const uint64_t *kin, const uint32_t *vin, const std::vector<uint64_t> &src, RadixBufs b, int first,
+                  uint64_t n, const std::vector<uint64_t> &seg, uint64_t *cuts, cudaStream_t s, uint64_t *rounds) {
+  int c = -1;
+  std::vector<uint64_t> cur = seg, from = src;
   while (cur.size() > 2) {  // more than one segment
+    const int o = c < 0 ? first : 1 - c;
     MergeRound r{};
-    r.kin = b.keys[c];
-    r.vin = b.vals[c];
-    r.kout = b.keys[1 - c];
-    r.vout = b.vals[1 - c];
+    r.kin = c < 0 ? kin : b.keys[c];
+    r.vin = c < 0 ? vin : b.vals[c];
+    r.kout = b.keys[o];
+    r.vout = b.vals[o];
     r.n = n;
     r.nseg = (uint32_t)(cur.size() - 1);
     for (size_t i = 0; i < cur.size(); ++i) r.seg[i] = cur[i];
+    for (size_t i = 0; i < from.size(); ++i) r.src[i] = from[i];
     const unsigned grid = (unsigned)((n + kMergeTile - 1) / kMergeTile);
     merge_cuts_kernel<<<(grid + 1 + 255) / 256, 256, 0, s>>>(r, cuts, (uint64_t)grid + 1);
     merge_round_kernel<<<grid, kMergeThreads, 0, s>>>(r, cuts);
     std::vector<uint64_t> nx;
     for (uint32_t q = 0; 2 * q < r.nseg; ++q) nx.push_back(cur[2 * q]);
+    from = nx;
     nx.push_back(n);
     cur.swap(nx);
-    c = 1 - c;
+    c = o;
     *rounds += 1;
   }
   return c;
@@ -520,7 +534,10 @@ struct MergePass : ExKernel {
     const size_t e = p % S;
     if (!ev0.empty()) VX_CUDA_TRY(cudaEventRecord(ev0[e], s));
     uint64_t rounds = 0;
-    result_buf[e] = merge_enqueue(bufs(slot), n, segments_of(lens), cuts(slot), s, &rounds);
+    const std::vector<uint64_t> seg = segments_of(lens);
+    const RadixBufs b = bufs(slot);
+    result_buf[e] = std::max(0, merge_enqueue(b.keys[0], b.vals[0], {seg.begin(), seg.end() - 1}, b, 1, n, seg,
+                                              cuts(slot), s, &rounds));
     VX_CUDA_TRY(cudaGetLastError());
     if (!ev1.empty()) VX_CUDA_TRY(cudaEventRecord(ev1[e], s));
     rounds_pairs += rounds * n;
@@ -541,6 +558,118 @@ struct MergePass : ExKernel {
       d2h.push_back({b.keys[c], out_keys + off, 8 * n});
       d2h.push_back({b.vals[c], out_vals + off, 4 * n});
     }
+    return VX_OK;
+  }
+};
+
+// ------------------------------------------------------------------ resident pairs
+// When the arena holds all pairs beside the passes' slots, they are loaded into
+// it once and stay: the input's own runs are found while the chunks arrive (or
+// the chunks are sorted into runs where they are), the cuts search HBM, and the
+// merge pass reads the runs' segments in place.  The pairs cross the link once
+// each way, in copies of whole chunks.  60M pairs in 64 runs (720 MB) under 1
+// GiB: 14.2 ms with the keys loaded to find the runs and the pairs again in 64
+// unaligned pieces a partition, 9.3 ms now, of which the merge rounds take 4.9.
+
+// the sorted chunk in buffer 0, wherever its radix sort left it
+__global__ void rx_home_kernel(RadixBufs b, const RadixState *st, uint64_t n) {
+  if (!st->cur[8]) return;
+  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+    b.keys[0][i] = b.keys[1][i];
+    b.vals[0][i] = b.vals[1][i];
+  }
+}
+
+struct ResidentRunPass : ExKernel {
+  vx_ctx *ctx;
+  const uint64_t *keys;
+  const uint32_t *vals;
+  uint64_t n, R;
+  uint64_t *rk;  // the resident pairs
+  uint32_t *rv;
+  bool load = true, sort = false;
+  int S;
+  unsigned long long *d_cnt = nullptr;  // find runs: descents
+  uint64_t *d_pos = nullptr;
+  uint64_t *d_fences = nullptr;  // sort: run it's at it * fences_per_run
+  uint64_t fences_per_run = 0, pass_pairs = 0;
+
+  uint64_t size() override { return (n + R - 1) / R; }
+  uint64_t rows(uint64_t it) const { return std::min(R, n - it * R); }
+  int n_slots() override { return S; }
+  int max_in_flight() override { return S; }
+  uint64_t kb() const { return (8 * R + 255) & ~255ull; }
+  uint64_t vb() const { return (4 * R + 255) & ~255ull; }
+  uint64_t slot_bytes() override { return sort ? kb() + vb() + radix_temp_bytes(R) : 256; }
+  void inputs(uint64_t it, char *, std::vector<CopyOp> &h2d) override {
+    if (!load) return;
+    h2d.push_back({keys + it * R, rk + it * R, 8 * rows(it)});
+    h2d.push_back({vals + it * R, rv + it * R, 4 * rows(it)});
+  }
+  vx_status kernel(char *slot, uint64_t it, cudaStream_t s) override {
+    const uint64_t m = rows(it);
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((m + 255) / 256, (uint64_t)ctx->num_sms * 8));
+    if (!sort) {  // the chunk's first row is compared with the row before it, which is there already
+      const uint64_t r0 = it ? it * R - 1 : 0;
+      descent_kernel<<<grid, 256, 0, s>>>(rk + r0, m + (it ? 1 : 0), r0, d_cnt, d_pos, kMaxRuns);
+      VX_CUDA_TRY(cudaGetLastError());
+      return VX_OK;
+    }
+    RadixBufs b;
+    b.keys[0] = rk + it * R;
+    b.vals[0] = rv + it * R;
+    b.keys[1] = (uint64_t *)slot;
+    b.vals[1] = (uint32_t *)(slot + kb());
+    char *temp = slot + kb() + vb();
+    VX_TRY(radix_sort_enqueue(b, m, temp, s, ctx->num_sms, 8, ctx->cfg.lookback_spin_limit));
+    rx_home_kernel<<<grid, 256, 0, s>>>(b, radix_state_of(temp), m);
+    const uint64_t nf = (m + kFenceStride - 1) / kFenceStride;
+    run_fences_kernel<<<(unsigned)std::max<uint64_t>(1, std::min<uint64_t>((nf + 255) / 256, 1024)), 256, 0, s>>>(
+        b.keys[0], nullptr, nullptr, m, d_fences + it * fences_per_run);
+    VX_CUDA_TRY(cudaGetLastError());
+    return radix_publish_enqueue(temp, ctx->d_scalars + 64 + (it % S), s);
+  }
+  bool has_outputs() override { return sort; }  // nothing is stored: the sort's outcome is read
+  vx_status outputs(uint64_t it, char *, std::vector<CopyOp> &) override {
+    const uint64_t word = ((volatile uint64_t *)ctx->h_scalars)[64 + (it % S)];
+    if (word >> 16 & 1) {
+      set_error("radix sort of run %llu: a look-back wait gave up", (unsigned long long)it);
+      return VX_E_TIMEOUT;
+    }
+    pass_pairs += rows(it) * ((word >> 8) & 0xFF);
+    return VX_OK;
+  }
+};
+
+struct ResidentMergePass : MergePass {
+  const uint64_t *rk;
+  const uint32_t *rv;
+  std::vector<uint64_t> only;  // per slot: where a partition of one segment starts (else ~0)
+  void inputs(uint64_t, char *, std::vector<CopyOp> &) override {}
+  vx_status kernel(char *slot, uint64_t p, cudaStream_t s) override {
+    std::vector<uint64_t> seg{0}, src;
+    for (uint32_t r = 0; r < N; ++r)
+      if (const uint64_t l = seg_len(p, r)) {
+        src.push_back(run_off[r] + cut[p * N + r]);
+        seg.push_back(seg.back() + l);
+      }
+    const size_t e = p % S;
+    if (!ev0.empty()) VX_CUDA_TRY(cudaEventRecord(ev0[e], s));
+    uint64_t rounds = 0;
+    result_buf[e] = merge_enqueue(rk, rv, src, bufs(slot), 0, seg.back(), seg, cuts(slot), s, &rounds);
+    only[e] = result_buf[e] < 0 && !src.empty() ? src[0] : 0;
+    VX_CUDA_TRY(cudaGetLastError());
+    if (!ev1.empty()) VX_CUDA_TRY(cudaEventRecord(ev1[e], s));
+    rounds_pairs += rounds * seg.back();
+    return VX_OK;
+  }
+  vx_status outputs(uint64_t p, char *slot, std::vector<CopyOp> &d2h) override {
+    const int c = result_buf[p % S];
+    const RadixBufs b = bufs(slot);
+    const uint64_t n = part_len(p), off = part_off(p);
+    if (!n) return VX_OK;
+    d2h.push_back({c < 0 ? rk + only[p % S] : b.keys[c], out_keys + off, 8 * n});
+    d2h.push_back({c < 0 ? rv + only[p % S] : b.vals[c], out_vals + off, 4 * n});
     return VX_OK;
   }
 };
@@ -583,6 +712,172 @@ vx_status exact_cuts(vx_ctx *ctx, const uint64_t *keys, const std::vector<uint64
   return VX_OK;
 }
 
+// slots of fewer pairs than this are not worth keeping the pairs resident
+constexpr uint64_t kMinResidentRows = 1 << 18;
+
+// Whether a few adjacent pairs already show an input of far more than kMaxRuns
+// runs (a sixteenth of them descending)
+bool clearly_unsorted(const uint64_t *keys, uint64_t n) {
+  const uint64_t ns = std::min<uint64_t>(1024, n - 1);
+  uint64_t desc = 0;
+  for (uint64_t j = 0; j < ns; ++j) {
+    const uint64_t i = 1 + (uint64_t)((unsigned __int128)(0x9E3779B97F4A7C15ull * (j + 1)) * (n - 1) >> 64);
+    desc += keys[i] < keys[i - 1];
+  }
+  return n > 16 * kMaxRuns && desc * 16 >= ns;
+}
+
+// The merge plan with resident pairs; *done = false: they do not fit.
+vx_status resident_merge_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals, uint64_t n, uint64_t *out_keys,
+                              uint32_t *out_vals, const vx_sort_opts &o, vx_sort_stats &ss, bool *done) {
+  *done = false;
+  const int S = std::max(2, ctx->cfg.n_slots);
+  const uint64_t avail = ctx->arena.largest_free();
+  const uint64_t kb = (8 * n + 255) & ~255ull, vb = (4 * n + 255) & ~255ull;
+  const uint64_t fence_words = n / kFenceStride + 4 * kMaxRuns + 8;  // every run's, their starts and offsets
+  const uint64_t fixed = kb + vb + 8 * fence_words + 8 * (kMaxRuns + 1) + (4 << 20);  // and the cuts' scratch
+  if (fixed >= avail) return VX_OK;
+  const uint64_t left = avail - fixed;
+  // merge slots: 24 bytes a pair and the cuts; chunks that are sorted in place: 12.5
+  const uint64_t cap2 = (uint64_t)((double)left / (S * 24.1) * 0.98);
+  uint64_t R = std::min<uint64_t>((uint64_t)((double)left / (S * (12.0 + 256.0 * 8 / kRxTile)) * 0.95),
+                                  std::max<uint64_t>(n / 8, 1 << 20));
+  R = std::min<uint64_t>(R, kPipelineRows) / kRxTile * kRxTile;
+  if (cap2 < kMinResidentRows || R < kMinResidentRows || (n + R - 1) / R > kMaxRuns) return VX_OK;
+  // partitions small enough that the first store starts early
+  uint64_t P = o.n_partitions > 0 ? (uint64_t)o.n_partitions
+                                  : std::max<uint64_t>((n + cap2 - 1) / cap2, std::min<uint64_t>(n >> 22, 64));
+  P = std::max<uint64_t>(P, 1);
+  if ((n + P - 1) / P > cap2) return VX_OK;
+  if (8 * P * (kMaxRuns + 4) > (4 << 20)) return VX_OK;
+  DevBuf mem;
+  mem.arena = &ctx->arena;
+  mem.p = ctx->arena.alloc(kb + vb + 8 * fence_words + 8 * (kMaxRuns + 1));
+  if (!mem.p) return VX_OK;
+  uint64_t *rk = mem.as<uint64_t>();
+  uint32_t *rv = (uint32_t *)(mem.as<char>() + kb);
+  uint64_t *d_fences = (uint64_t *)(mem.as<char>() + kb + vb);
+  unsigned long long *d_cnt = (unsigned long long *)(d_fences + fence_words);
+  cudaStream_t s = ctx->s_compute;
+  const double t0 = now_ms();
+  ResidentRunPass rp;
+  rp.ctx = ctx;
+  rp.keys = keys;
+  rp.vals = vals;
+  rp.n = n;
+  rp.rk = rk;
+  rp.rv = rv;
+  rp.S = S;
+  bool nat = false;
+  std::vector<uint64_t> run_off{0}, fence_start;
+  if (o.runs_mode == 0 && !clearly_unsorted(keys, n)) {
+    VX_CUDA_TRY(cudaMemsetAsync(d_cnt, 0, 8, s));
+    rp.R = std::min<uint64_t>(std::max<uint64_t>(n / 16, 1 << 20), kPipelineRows) / kRxTile * kRxTile;
+    rp.d_cnt = d_cnt;
+    rp.d_pos = (uint64_t *)d_cnt + 1;
+    ExecStats es;
+    VX_TRY(run_pipeline(ctx, rp, &es));
+    ss.bytes_h2d += es.bytes_h2d;
+    ss.kernel_launches += es.kernel_launches;
+    rp.load = false;
+    std::vector<uint64_t> h(kMaxRuns + 1);
+    VX_CUDA_TRY(cudaMemcpyAsync(h.data(), d_cnt, 8 * h.size(), cudaMemcpyDeviceToHost, s));
+    VX_CUDA_TRY(cudaStreamSynchronize(s));
+    nat = h[0] + 1 <= kMaxRuns;
+    if (nat) {
+      std::sort(h.begin() + 1, h.begin() + 1 + h[0]);
+      run_off.insert(run_off.end(), h.begin() + 1, h.begin() + 1 + h[0]);
+    }
+  }
+  if (nat) {
+    run_off.push_back(n);
+    const uint32_t N = (uint32_t)run_off.size() - 1;
+    uint64_t nf = 0, mx_nf = 0;
+    for (uint32_t r = 0; r < N; ++r) {
+      const uint64_t f = (run_off[r + 1] - run_off[r] + kFenceStride - 1) / kFenceStride;
+      fence_start.push_back(nf);
+      nf += f;
+      mx_nf = std::max(mx_nf, f);
+    }
+    uint64_t *d_off = d_fences + nf, *d_fs = d_off + N + 1;
+    VX_CUDA_TRY(cudaMemcpyAsync(d_off, run_off.data(), 8 * (N + 1), cudaMemcpyHostToDevice, s));
+    VX_CUDA_TRY(cudaMemcpyAsync(d_fs, fence_start.data(), 8 * N, cudaMemcpyHostToDevice, s));
+    const dim3 grid((unsigned)std::max<uint64_t>(1, std::min<uint64_t>((mx_nf + 255) / 256, 256)), N);
+    natural_fences_kernel<<<grid, 256, 0, s>>>(rk, d_off, d_fs, d_fences);
+    VX_CUDA_TRY(cudaGetLastError());
+    ss.natural_runs = 1;
+  } else {
+    rp.sort = true;
+    rp.R = R;
+    rp.d_fences = d_fences;
+    rp.fences_per_run = (R + kFenceStride - 1) / kFenceStride;
+    ExecStats es;
+    VX_TRY(run_pipeline(ctx, rp, &es));
+    VX_CUDA_TRY(cudaStreamSynchronize(s));
+    ss.bytes_h2d += es.bytes_h2d;
+    ss.kernel_launches += es.kernel_launches * 13;  // radix sort (10), home, fences, publish
+    ss.ms_sort_kernel += es.ms_kernel;
+    ss.radix_pass_pairs += rp.pass_pairs;
+    for (uint64_t at = 0; at < n; at += R) {
+      fence_start.push_back(at / R * rp.fences_per_run);
+      run_off.push_back(std::min(at + R, n));
+    }
+  }
+  const uint32_t N = (uint32_t)run_off.size() - 1;
+  ss.n_runs = N;
+  ss.ms_partition += now_ms() - t0;
+
+  const double ts = now_ms();
+  std::vector<uint64_t> ranks, inner;
+  for (uint64_t p = 1; p < P; ++p) ranks.push_back(p * n / P);
+  VX_TRY(exact_cuts(ctx, rk, run_off, fence_start, d_fences, ranks, &inner));
+  ResidentMergePass mp;
+  mp.ctx = ctx;
+  mp.rk = rk;
+  mp.rv = rv;
+  mp.run_off = run_off;
+  mp.N = N;
+  mp.P = (uint32_t)P;
+  mp.cut.assign((P + 1) * N, 0);
+  for (uint64_t p = 1; p < P; ++p)
+    for (uint32_t r = 0; r < N; ++r) mp.cut[p * N + r] = inner[(p - 1) * N + r];
+  for (uint32_t r = 0; r < N; ++r) mp.cut[P * N + r] = run_off[r + 1] - run_off[r];
+  ss.max_partition = ss.min_partition = mp.part_len(0);
+  for (uint64_t p = 1; p < P; ++p) {
+    ss.max_partition = std::max<uint64_t>(ss.max_partition, mp.part_len(p));
+    ss.min_partition = std::min<uint64_t>(ss.min_partition, mp.part_len(p));
+  }
+  ss.ms_sample += now_ms() - ts;
+  ss.n_partitions = (uint32_t)P;
+  ss.imbalance = (double)ss.max_partition / ((double)n / P);
+
+  const double tq = now_ms();
+  mp.cap = (ss.max_partition + kMergeTile - 1) / kMergeTile * kMergeTile;
+  mp.S = std::max<int>(2, (int)std::min<uint64_t>(S, ctx->arena.largest_free() / ((mp.slot_bytes() + 255) & ~255ull)));
+  mp.result_buf.assign(mp.S, 0);
+  mp.only.assign(mp.S, 0);
+  mp.out_keys = out_keys;
+  mp.out_vals = out_vals;
+  if (ctx->cfg.sched == VX_SCHED_IMMEDIATE) {
+    mp.ev0.resize(mp.S);
+    mp.ev1.resize(mp.S);
+    for (int i = 0; i < mp.S; ++i) {
+      VX_CUDA_TRY(cudaEventCreate(&mp.ev0[i]));
+      VX_CUDA_TRY(cudaEventCreate(&mp.ev1[i]));
+    }
+  }
+  ExecStats es;
+  VX_TRY(run_pipeline(ctx, mp, &es));
+  ss.bytes_d2h += es.bytes_d2h;
+  ss.kernel_launches += es.kernel_launches;
+  ss.ms_merge_kernel += mp.ms_merge;
+  ss.merge_pass_pairs += mp.rounds_pairs;
+  ss.slot_pairs = mp.cap;
+  ss.ms_sort += now_ms() - tq;
+  *done = true;
+  return VX_OK;
+}
+
 }  // namespace
 
 // The merge plan of vx_sort.  When a sample of adjacent pairs suggests the
@@ -596,6 +891,11 @@ vx_status merge_sort_plan(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
   const int S = std::max(2, ctx->cfg.n_slots);
   ss.plan = VX_SORT_MERGE;
   if (n == 0) return VX_OK;
+  if (!o.max_slot_pairs) {
+    bool done = false;
+    VX_TRY(resident_merge_sort(ctx, keys, vals, n, out_keys, out_vals, o, ss, &done));
+    if (done) return VX_OK;
+  }
   std::vector<uint64_t> run_off, fence_start;
   DevBuf fb;
   fb.arena = &ctx->arena;
@@ -887,7 +1187,9 @@ VX_API vx_status vx_merge_runs(vx_ctx *ctx, const uint64_t *keys, const uint32_t
   VX_CUDA_TRY(cudaMemcpyAsync(b.keys[0], keys, 8 * n, cudaMemcpyHostToDevice, s));
   VX_CUDA_TRY(cudaMemcpyAsync(b.vals[0], vals, 4 * n, cudaMemcpyHostToDevice, s));
   uint64_t rounds = 0;
-  const int c = merge_enqueue(b, n, segments_of(lens), (uint64_t *)(buf.as<char>() + 2 * kb + 2 * vb), s, &rounds);
+  const std::vector<uint64_t> seg = segments_of(lens);
+  const int c = std::max(0, merge_enqueue(b.keys[0], b.vals[0], {seg.begin(), seg.end() - 1}, b, 1, n, seg,
+                                          (uint64_t *)(buf.as<char>() + 2 * kb + 2 * vb), s, &rounds));
   VX_CUDA_TRY(cudaGetLastError());
   VX_CUDA_TRY(cudaMemcpyAsync(out_keys, b.keys[c], 8 * n, cudaMemcpyDeviceToHost, s));
   VX_CUDA_TRY(cudaMemcpyAsync(out_vals, b.vals[c], 4 * n, cudaMemcpyDeviceToHost, s));
