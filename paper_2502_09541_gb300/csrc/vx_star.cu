@@ -370,6 +370,14 @@ __device__ __forceinline__ void star_eval4(const ChunkParams &p, uint64_t r0, co
   star_probe_dims<kN>(p, vals, alive, g);
 }
 
+// sums over the warp, complete in lane 0
+__device__ __forceinline__ void warp_total(unsigned long long &v, uint32_t &c) {
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (!c) return;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+}
+
 template <bool kSmem, bool kSplit, int kV, class Vals, class Tile>
 __device__ __forceinline__ void star_rows4(const ChunkParams &p, uint64_t r0, const Vals &vals,
                                            unsigned long long *ssum, unsigned long long *scnt,
@@ -387,6 +395,8 @@ __device__ __forceinline__ void star_rows4(const ChunkParams &p, uint64_t r0, co
     for (int j = 0; j < kN; ++j)
       if (alive[j]) st->e[atomicAdd(&st->n, 1u)] = make_uint2((uint32_t)row_of(r0, j), g[j]);
   } else {
+    unsigned long long tv = 0;  // one group: the warp's total, added once
+    uint32_t tc = 0;
 #pragma unroll
     for (int j = 0; j < kN; ++j) {
       if (!alive[j]) continue;
@@ -397,12 +407,22 @@ __device__ __forceinline__ void star_rows4(const ChunkParams &p, uint64_t r0, co
                         : p.agg_slot[1] >= 0 ? vals(p.agg_slot[1], j)
                                              : load_role(p, p.agg_b_role, row_of(r0, j));
       const int64_t v = p.agg_op == VX_AGG_SUM ? a : p.agg_op == VX_AGG_MUL ? a * b : p.agg_op == VX_AGG_SUB ? a - b : 0;
-      if (kSmem) {
+      if (p.n_groups == 1) {
+        tv += (unsigned long long)v;
+        ++tc;
+      } else if (kSmem) {
         atomicAdd(&ssum[g[j]], (unsigned long long)v);
         atomicAdd(&scnt[g[j]], 1ull);
       } else {
         atomicAdd(&p.g_sum[g[j]], (unsigned long long)v);
         atomicAdd(&p.g_cnt[g[j]], 1ull);
+      }
+    }
+    if (p.n_groups == 1) {  // every thread of the block gets here
+      warp_total(tv, tc);
+      if ((threadIdx.x & 31) == 0 && tc) {
+        atomicAdd(kSmem ? &ssum[0] : &p.g_sum[0], tv);
+        atomicAdd(kSmem ? &scnt[0] : &p.g_cnt[0], (unsigned long long)tc);
       }
     }
   }
@@ -600,7 +620,8 @@ __global__ void __launch_bounds__(256, 6) star_bulk_kernel(const ChunkParams p, 
     if constexpr (kSplit) {
       if (ok) star_eval4<1>(p, r0, vals, alive, g);
     } else {
-      if (ok) star_rows4<kSmem, false, 1>(p, r0, vals, ssum, scnt, surv, static_cast<SurvTile *>(nullptr));
+      // (a warp's lanes evaluate together or not at all: the totals use its votes)
+      if (__all_sync(0xffffffffu, ok)) star_rows4<kSmem, false, 1>(p, r0, vals, ssum, scnt, surv, static_cast<SurvTile *>(nullptr));
     }
     uint32_t b[4] = {0, 0, 0, 0}, wtot = 0;
     if constexpr (kSplit) {
@@ -824,6 +845,10 @@ __global__ void __launch_bounds__(256) star_split_kernel(const ChunkParams p) {
 // mapped host memory with one independent load per survivor in flight, and
 // aggregated into the group accumulators.  A chunk whose survivors did not
 // fit the list is not aggregated at all: it is flagged for an exact rerun.
+// A plan without group keys has one accumulator: each block adds its total to it
+// once.  (A 64-bit shared-memory add per survivor made the block's survivors
+// queue for one word: 30 us a chunk of 9,300 survivors beside the next chunk's
+// copy, 13 now.)
 template <bool kSmem>
 __global__ void __launch_bounds__(256) star_gather_kernel(const ChunkParams p) {
   extern __shared__ unsigned long long sacc[];
@@ -836,6 +861,9 @@ __global__ void __launch_bounds__(256) star_gather_kernel(const ChunkParams p) {
     }
     return;
   }
+  const bool one = p.n_groups == 1;
+  unsigned long long tv = 0;
+  uint32_t tc = 0;
   if (kSmem) {
     for (uint32_t g = threadIdx.x; g < 2 * p.n_groups; g += blockDim.x) sacc[g] = 0;
     __syncthreads();
@@ -845,12 +873,22 @@ __global__ void __launch_bounds__(256) star_gather_kernel(const ChunkParams p) {
     const int64_t a = p.agg_a_role >= 0 ? load_role(p, p.agg_a_role, e.x) : 0;
     const int64_t b = p.agg_b_role >= 0 ? load_role(p, p.agg_b_role, e.x) : 0;
     const int64_t v = p.agg_op == VX_AGG_SUM ? a : p.agg_op == VX_AGG_MUL ? a * b : p.agg_op == VX_AGG_SUB ? a - b : 0;
-    if (kSmem) {
+    if (one) {
+      tv += (unsigned long long)v;
+      ++tc;
+    } else if (kSmem) {
       atomicAdd(&ssum[e.y], (unsigned long long)v);
       atomicAdd(&scnt[e.y], 1ull);
     } else {
       atomicAdd(&p.g_sum[e.y], (unsigned long long)v);
       atomicAdd(&p.g_cnt[e.y], 1ull);
+    }
+  }
+  if (one) {
+    warp_total(tv, tc);
+    if ((threadIdx.x & 31) == 0 && tc) {
+      atomicAdd(kSmem ? &ssum[0] : &p.g_sum[0], tv);
+      atomicAdd(kSmem ? &scnt[0] : &p.g_cnt[0], (unsigned long long)tc);
     }
   }
   if (kSmem) {
