@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <cstdarg>
 #include <cstdio>
+#include <thread>
 
 #include "vx_internal.h"
 
@@ -20,6 +21,11 @@ void clear_error() { g_err[0] = 0; }
 double now_ms() {
   using namespace std::chrono;
   return duration<double, std::milli>(steady_clock::now().time_since_epoch()).count();
+}
+
+void poll_pause(double since) {
+  if (now_ms() - since < kSpinMs) std::this_thread::yield();
+  else std::this_thread::sleep_for(std::chrono::microseconds(10));
 }
 
 // ------------------------------------------------------------------ arena

@@ -69,6 +69,7 @@ struct CudaDev {
   double t_origin;
   DevBuf *ring;
   std::vector<CopyOp> ops;
+  double last_step = 0;  // when a step was issued or found complete last
 
   char *slot(int s) const { return base + (uint64_t)s * slot_bytes; }
   static int state(cudaEvent_t e) {
@@ -80,6 +81,7 @@ struct CudaDev {
   }
   bool has_outputs() { return k.has_outputs(); }
   vx_status load(uint64_t it, int s) {
+    last_step = vx::now_ms();
     SlotState &sl = es.s[s];
     ops.clear();
     k.inputs(it, slot(s), ops);
@@ -100,6 +102,7 @@ struct CudaDev {
   }
   int kernel_state(int s) { return state(es.s[s].ev_k); }
   vx_status retire(uint64_t it, int s) {
+    last_step = vx::now_ms();
     SlotState &sl = es.s[s];
     float ms = 0;
     if (cudaEventElapsedTime(&ms, sl.ev_k0, sl.ev_k) == cudaSuccess) st->ms_kernel += ms;
@@ -124,6 +127,7 @@ struct CudaDev {
   }
   int store_state(int s) { return state(es.s[s].ev_out); }
   vx_status stored(uint64_t, int s) {
+    last_step = vx::now_ms();
     if (tl) {  // this chunk's row is the last one recorded so far (chunks retire in order)
       float *row = &ctx->timeline[ctx->timeline.size() - VX_TIMELINE_COLS];
       row[6] = since(es.ref, es.s[s].ev_d0);
@@ -140,7 +144,7 @@ struct CudaDev {
     return VX_E_TIMEOUT;
   }
   double now_ms() { return vx::now_ms(); }
-  void pause() { std::this_thread::sleep_for(std::chrono::microseconds(10)); }
+  void pause() { poll_pause(last_step); }
 };
 
 }  // namespace

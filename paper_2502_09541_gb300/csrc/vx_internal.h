@@ -168,6 +168,12 @@ vx_status check_ctx(vx_ctx *ctx);
 const Column *get_col(vx_ctx *ctx, int32_t id, int32_t want_dtype /* -1 any */);
 double now_ms();
 
+// Between polls of work that finishes within microseconds: yields for the first
+// kSpinMs after `since` (a sleep of 10 us takes 60-70 us here, twice what a
+// small chunk's copy takes), then sleeps.
+constexpr double kSpinMs = 1.0;
+void poll_pause(double since_ms);
+
 // ------------------------------------------------------------------ executor
 // A host->device or device->host copy of one extent.
 struct CopyOp {

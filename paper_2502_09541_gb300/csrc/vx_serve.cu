@@ -221,7 +221,7 @@ static vx_status cycle(ServeEngine &e, bool *did) {
         set_error("serving: wait limit expired");
         return VX_E_TIMEOUT;
       }
-      std::this_thread::sleep_for(std::chrono::microseconds(10));
+      poll_pause(t_w);
     }
   }
   const uint64_t cr = serve_chunk_rows(e);
@@ -356,6 +356,7 @@ static void reap(ServeEngine &e) {
 static void engine_loop(ServeEngine *e) {
   cudaSetDevice(e->ctx->device);
   std::unique_lock<std::mutex> lk(e->mu);
+  double t_did = now_ms();  // the last cycle
   while (!e->stop) {
     admit(*e);
     bool did = false;
@@ -374,12 +375,13 @@ static void engine_loop(ServeEngine *e) {
     }
     reap(*e);
     e->cv_done.notify_all();
+    if (did) t_did = now_ms();
     if (!did) {
       if (e->pending.empty() && e->active.empty())
         e->cv.wait_for(lk, std::chrono::milliseconds(5));
       else if (!did) {
         lk.unlock();
-        std::this_thread::sleep_for(std::chrono::microseconds(20));
+        poll_pause(t_did);
         lk.lock();
       }
     }

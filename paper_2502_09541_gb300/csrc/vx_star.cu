@@ -1403,10 +1403,14 @@ vx_status build_dim_table(vx_ctx *ctx, const DimSpec &d, BuiltDim *out, uint32_t
   return VX_OK;
 }
 
-vx_status check_err_word(vx_ctx *ctx, const uint32_t *d_err) {
-  uint32_t e = 0;
-  VX_CUDA_TRY(cudaMemcpyAsync(&e, d_err, 4, cudaMemcpyDeviceToHost, ctx->s_compute));
-  VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
+// Words of the context's page-locked block that a star call reads small results
+// through (a copy into pageable memory costs a staging round trip): the sampled
+// predicate count, the error word, then the accumulators of up to kPinnedGroups
+// groups.
+constexpr int kPinSample = 1000, kPinErr = 1001, kPinAcc = 1024;
+constexpr uint64_t kPinnedGroups = (vx_ctx::kScalars - kPinAcc) / 2;
+
+static vx_status err_status(uint32_t e) {
   if (e & ERR_DUPKEY) {
     set_error("duplicate key on the build side");
     return VX_E_DUPKEY;
@@ -1428,6 +1432,13 @@ vx_status check_err_word(vx_ctx *ctx, const uint32_t *d_err) {
     return VX_E_TIMEOUT;
   }
   return VX_OK;
+}
+
+vx_status check_err_word(vx_ctx *ctx, const uint32_t *d_err) {
+  uint32_t e = 0;
+  VX_CUDA_TRY(cudaMemcpyAsync(&e, d_err, 4, cudaMemcpyDeviceToHost, ctx->s_compute));
+  VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
+  return err_status(e);
 }
 
 // ------------------------------------------------------------------ star ExKernel
@@ -1861,6 +1872,7 @@ vx_status run_star(vx_ctx *ctx, const vx_plan *plan, vx_result *out, bool use_re
 
   // ---- dimension tables (Section 7.1: filtered, hashed, kept on the device)
   std::vector<std::shared_ptr<ResidentHT>> tables(plan->n_dims);
+  bool built = false;
   for (int d = 0; d < plan->n_dims; ++d) {
     std::string sig = dim_signature(dspec[d]);
     auto it = use_resident ? ctx->resident.find(sig) : ctx->resident.end();
@@ -1871,11 +1883,14 @@ vx_status run_star(vx_ctx *ctx, const vx_plan *plan, vx_result *out, bool use_re
     auto t = std::make_shared<ResidentHT>();
     VX_TRY(build_dim_table(ctx, dspec[d], &t->dim, d_err, d_cnt + d));
     tables[d] = t;
+    built = true;
   }
   {
     uint64_t passed[VX_MAX_DIMS] = {0};
-    VX_CUDA_TRY(cudaMemcpyAsync(passed, d_cnt, 8 * VX_MAX_DIMS, cudaMemcpyDeviceToHost, ctx->s_compute));
-    VX_TRY(check_err_word(ctx, d_err));
+    if (built) {  // the builds' row counts and errors
+      VX_CUDA_TRY(cudaMemcpyAsync(passed, d_cnt, 8 * VX_MAX_DIMS, cudaMemcpyDeviceToHost, ctx->s_compute));
+      VX_TRY(check_err_word(ctx, d_err));
+    }
     for (int d = 0; d < plan->n_dims; ++d) {
       if (!tables[d]->built) {
         tables[d]->dim.passed = passed[d];
@@ -1910,9 +1925,9 @@ vx_status run_star(vx_ctx *ctx, const vx_plan *plan, vx_result *out, bool use_re
     sp.out = (unsigned long long *)(d_cnt + 15);
     sample_preds_kernel<<<16, 256, 0, ctx->s_compute>>>(sp);
     VX_CUDA_TRY(cudaGetLastError());
-    uint64_t hit = 0;
-    VX_CUDA_TRY(cudaMemcpyAsync(&hit, d_cnt + 15, 8, cudaMemcpyDeviceToHost, ctx->s_compute));
+    VX_CUDA_TRY(cudaMemcpyAsync(ctx->h_scalars + kPinSample, d_cnt + 15, 8, cudaMemcpyDeviceToHost, ctx->s_compute));
     VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
+    const uint64_t hit = ((volatile uint64_t *)ctx->h_scalars)[kPinSample];
     est *= (double)hit / (double)sp.n_samples;
   }
   qs.est_selectivity = est;
@@ -2129,8 +2144,16 @@ vx_status run_star(vx_ctx *ctx, const vx_plan *plan, vx_result *out, bool use_re
     }
   }
   if (!ge && n_rows) VX_TRY(run_pipeline(ctx, ek, &es));
-  VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
-  VX_TRY(check_err_word(ctx, res_err));
+  // the error word and the accumulators, behind the last kernel
+  std::vector<uint64_t> far(G > kPinnedGroups ? 2 * G : 0);
+  volatile uint64_t *h = G > kPinnedGroups ? far.data() : ctx->h_scalars + kPinAcc;
+  auto read_back = [&]() -> vx_status {
+    VX_CUDA_TRY(cudaMemcpyAsync(ctx->h_scalars + kPinErr, res_err, 4, cudaMemcpyDeviceToHost, ctx->s_compute));
+    VX_CUDA_TRY(cudaMemcpyAsync((void *)h, res_acc, 16 * G, cudaMemcpyDeviceToHost, ctx->s_compute));
+    VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
+    return err_status((uint32_t)((volatile uint64_t *)ctx->h_scalars)[kPinErr]);
+  };
+  VX_TRY(read_back());
   uint32_t overflow_retries = 0;
   if (res_ovf) {  // chunks whose survivors outgrew the predicted list: rerun them exactly
     std::vector<unsigned int> fl(n_chunks);
@@ -2159,8 +2182,7 @@ vx_status run_star(vx_ctx *ctx, const vx_plan *plan, vx_result *out, bool use_re
       rk.surv_rows = 0;  // worst case: every row of the chunk
       ExecStats er;
       VX_TRY(run_pipeline(ctx, rk, &er));
-      VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
-      VX_TRY(check_err_word(ctx, res_err));
+      VX_TRY(read_back());
       es.bytes_h2d += er.bytes_h2d;
       overflow_retries = (uint32_t)rk.only.size();
       ek.launches += rk.launches;
@@ -2189,8 +2211,6 @@ vx_status run_star(vx_ctx *ctx, const vx_plan *plan, vx_result *out, bool use_re
   }
 
   // ---- results: non-empty groups in ascending id
-  std::vector<uint64_t> h(2 * G);
-  VX_CUDA_TRY(cudaMemcpy(h.data(), res_acc, 16 * G, cudaMemcpyDeviceToHost));
   uint64_t n_out = 0, surv = 0;
   vx_status st = VX_OK;
   for (uint64_t g = 0; g < G; ++g) {
