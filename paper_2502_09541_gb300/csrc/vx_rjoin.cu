@@ -145,34 +145,42 @@ struct RjAcc {
   uint32_t err;
 };
 
-// resident mode: the clustered chunk leaves its slot for the resident arrays
-// (build side: with its payloads in clustered order; probe side: with its rows)
+// resident mode, after a chunk's clustering: its buffer 1 is the resident
+// array, where the last executed pass of an odd number of them has left the
+// keys (and the probe side's rows); an even number left them in the slot.  The
+// build side's payloads follow in clustered order.
 __global__ void rj_keep_kernel(const RadixBufs b, const RadixState *st, int npass, uint64_t n, const uint64_t *pay,
-                               uint64_t *okeys, uint64_t *opay, uint32_t *orows, RjAcc *acc) {
+                               uint64_t *opay, RjAcc *acc) {
   const int c = st->cur[npass];
-  const uint64_t *k = b.keys[c];
-  const uint32_t *v = b.vals[c];
+  const uint64_t *k = c ? b.keys[1] : b.keys[0];
+  const uint32_t *v = c ? b.vals[1] : b.vals[0];
+  bool moved = false;
+  for (int q = 0; q < npass; ++q) moved = moved || !st->skip[q];
   if (st->err && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&acc->err, ERR_WAIT);
+  if (c && !opay) return;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    okeys[i] = k[i];
-    if (opay) opay[i] = pay[v[i]];
-    else orows[i] = v[i];
+    const uint32_t row = moved ? v[i] : (uint32_t)i;
+    if (!c) b.keys[1][i] = k[i];
+    if (opay) opay[i] = pay[row];
+    else b.vals[1][i] = row;
   }
 }
 
-// resident mode: where the runs of 2^shift groups start in a clustered chunk
-// (bnd[r] for r <= n_runs, by binary search: a run has hundreds of tuples, so
-// this reads far less than the keys)
-__global__ void rj_cuts_kernel(const RadixBufs b, const RadixState *st, int npass, uint32_t n, uint64_t mask, int shift,
-                               uint32_t n_runs, uint32_t *bnd) {
-  const uint64_t *k = b.keys[st->cur[npass]];
+// resident mode: where the runs of 2^shift groups start in each clustered chunk
+// of R tuples (chunk c: bnd[c * (n_runs + 1) + r] for r <= n_runs), by binary
+// search: a run has hundreds of tuples, so this reads far less than the keys
+__global__ void rj_cuts_kernel(const uint64_t *keys, uint64_t n, uint64_t R, uint64_t mask, int shift, uint32_t n_runs,
+                               uint32_t *bnd) {
+  const uint64_t r0 = blockIdx.y * R;
+  const uint64_t *k = keys + r0;
+  const uint32_t m = (uint32_t)(n - r0 < R ? n - r0 : R);
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r <= n_runs; r += gridDim.x * blockDim.x) {
-    uint32_t lo = 0, hi = n;
+    uint32_t lo = 0, hi = m;
     while (lo < hi) {
       const uint32_t mid = lo + (hi - lo) / 2;
       if ((k[mid] & mask) >> shift < r) lo = mid + 1; else hi = mid;
     }
-    bnd[r] = lo;
+    bnd[blockIdx.y * (n_runs + 1ull) + r] = lo;
   }
 }
 
@@ -419,12 +427,10 @@ struct RjPartitionPass : ExKernel {
   uint64_t *mid_keys;
   uint64_t *mid_pay;    // build side
   uint32_t *mid_rows;   // probe side
-  uint32_t *mid_bnd;    // chunk c at c * (2^bits + 1), or resident: at c * (n_runs + 1)
-  // resident: mid_* are device memory, the slot's results are copied there and
-  // the boundary arrays hold the starts of n_runs runs of 2^run_shift groups
+  uint32_t *mid_bnd;    // chunk c at c * (2^bits + 1)
+  // resident: mid_keys, mid_pay and mid_rows are device memory, which the
+  // clustering writes; the slot holds the other buffer
   bool resident = false;
-  uint32_t n_runs = 0;
-  int run_shift = 0;
   RjAcc *acc = nullptr;
   uint64_t size() override { return (n + R - 1) / R; }
   int n_slots() override { return S; }
@@ -436,7 +442,7 @@ struct RjPartitionPass : ExKernel {
   uint64_t bb() const { return (4 * G1() + 255) & ~255ull; }
   uint64_t cb() const { return (4 * ((G1() + kRjSeg - 1) / kRjSeg) + 255) & ~255ull; }
   uint64_t slot_bytes() override {
-    if (resident) return 2 * kb() + 2 * vb() + radix_temp_bytes(R) + (payload ? kb() : 0);
+    if (resident) return kb() + 2 * vb() + radix_temp_bytes(R) + (payload ? kb() : 0);
     return 2 * kb() + 2 * vb() + radix_temp_bytes(R) + bb() + cb() + (payload ? 2 * kb() : 0);
   }
   RadixBufs bufs(char *slot) const {
@@ -447,7 +453,16 @@ struct RjPartitionPass : ExKernel {
     b.vals[1] = (uint32_t *)(slot + 2 * kb() + vb());
     return b;
   }
-  char *temp(char *slot) const { return slot + 2 * kb() + 2 * vb(); }
+  // resident: [keys | rows | rows (build side) | temp | payloads]
+  RadixBufs resident_bufs(char *slot, uint64_t it) const {
+    RadixBufs b;
+    b.keys[0] = (uint64_t *)slot;
+    b.keys[1] = mid_keys + it * R;
+    b.vals[0] = (uint32_t *)(slot + kb());
+    b.vals[1] = payload ? (uint32_t *)(slot + kb() + vb()) : mid_rows + it * R;
+    return b;
+  }
+  char *temp(char *slot) const { return slot + (resident ? 1 : 2) * kb() + 2 * vb(); }
   uint32_t *bnd(char *slot) const { return (uint32_t *)(temp(slot) + radix_temp_bytes(R)); }
   uint32_t *carry(char *slot) const { return (uint32_t *)((char *)bnd(slot) + bb()); }
   uint64_t *pay_in(char *slot) const {
@@ -459,20 +474,20 @@ struct RjPartitionPass : ExKernel {
     if (payload) h2d.push_back({payload + it * R, pay_in(slot), 8 * rows(it)});
   }
   vx_status kernel(char *slot, uint64_t it, cudaStream_t s) override {
-    RadixBufs b = bufs(slot);
     const uint64_t m = rows(it);
-    rj_iota_kernel<<<grid_for(ctx, m, 256, 8), 256, 0, s>>>(b.vals[0], m);
-    VX_TRY(radix_sort_enqueue(b, m, temp(slot), s, ctx->num_sms, npass, ctx->cfg.lookback_spin_limit));
-    const RadixState *st = radix_state_of(temp(slot));
     if (resident) {
-      rj_cuts_kernel<<<grid_for(ctx, n_runs + 1, 256, 8), 256, 0, s>>>(b, st, npass, (uint32_t)m, (1ull << bits) - 1,
-                                                                       run_shift, n_runs, mid_bnd + it * (n_runs + 1));
-      rj_keep_kernel<<<grid_for(ctx, m, 256, 8), 256, 0, s>>>(b, st, npass, m, payload ? pay_in(slot) : nullptr,
-                                                              mid_keys + it * R, payload ? mid_pay + it * R : nullptr,
-                                                              payload ? nullptr : mid_rows + it * R, acc);
+      const RadixBufs rb = resident_bufs(slot, it);
+      VX_TRY(radix_sort_enqueue(rb, m, temp(slot), s, ctx->num_sms, npass, ctx->cfg.lookback_spin_limit, true));
+      rj_keep_kernel<<<grid_for(ctx, m, 256, 8), 256, 0, s>>>(rb, radix_state_of(temp(slot)), npass, m,
+                                                              payload ? pay_in(slot) : nullptr,
+                                                              payload ? mid_pay + it * R : nullptr, acc);
       VX_CUDA_TRY(cudaGetLastError());
       return VX_OK;
     }
+    RadixBufs b = bufs(slot);
+    rj_iota_kernel<<<grid_for(ctx, m, 256, 8), 256, 0, s>>>(b.vals[0], m);
+    VX_TRY(radix_sort_enqueue(b, m, temp(slot), s, ctx->num_sms, npass, ctx->cfg.lookback_spin_limit));
+    const RadixState *st = radix_state_of(temp(slot));
     VX_TRY(find_boundary_enqueue(ctx, b, st, npass, m, bits, bnd(slot), carry(slot), s));
     if (payload)
       rj_gather_kernel<<<grid_for(ctx, m, 256, 8), 256, 0, s>>>(b.vals[0], b.vals[1], st, npass, m, pay_in(slot),
@@ -635,7 +650,7 @@ struct RjResident {
     bytes = items + rj_items_bytes(n_runs, np);
     return bytes;
   }
-  static uint64_t slot_bytes(uint64_t R) { return 3 * (8 * R + 255) + 2 * (4 * R + 255) + radix_temp_bytes(R); }
+  static uint64_t slot_bytes(uint64_t R) { return 2 * (8 * R + 255) + 2 * (4 * R + 255) + radix_temp_bytes(R); }
 };
 
 // The join with both clustered tables kept in device memory.  Against host
@@ -675,18 +690,20 @@ vx_status radix_join_resident(vx_ctx *ctx, const Column *bk, const Column *bp, c
     pp.bits = bits;
     pp.npass = bits / 8;
     pp.S = std::max(2, ctx->cfg.n_slots);
+    pp.mid_bnd = nullptr;
     pp.mid_keys = (uint64_t *)(m + (side ? rs.bkeys : rs.akeys));
     pp.mid_pay = (uint64_t *)(m + rs.apay);
     pp.mid_rows = (uint32_t *)(m + rs.brows);
-    pp.mid_bnd = (uint32_t *)(m + (side ? rs.bbnd : rs.abnd));
     pp.resident = true;
-    pp.n_runs = n_runs;
-    pp.run_shift = run_shift;
     pp.acc = acc;
     ExecStats es;
     VX_TRY(run_pipeline(ctx, pp, &es));
+    const uint32_t chunks = side ? rs.NB : rs.NA;
+    rj_cuts_kernel<<<dim3((unsigned)grid_for(ctx, n_runs + 1, 256, 8), chunks), 256, 0, s>>>(
+        pp.mid_keys, n, R, (1ull << bits) - 1, run_shift, n_runs, (uint32_t *)(m + (side ? rs.bbnd : rs.abnd)));
+    VX_CUDA_TRY(cudaGetLastError());
     res.bytes_h2d += es.bytes_h2d;
-    res.kernel_launches += es.kernel_launches * (pp.npass + 5);
+    res.kernel_launches += es.kernel_launches * (pp.npass + 3) + 1;
     res.ms_kernel += es.ms_kernel;
   }
   res.ms_partition = res.ms_build = now_ms() - tp;

@@ -358,7 +358,7 @@ struct RxSweepSmem {
 template <int kT, int kI, class Off>
 __global__ void __launch_bounds__(kT, 2) rx_sweep(RadixBufs b, RadixState *st, int pass, uint64_t n,
                                                           const uint64_t *bases, unsigned int *tickets,
-                                                          unsigned long long *status) {
+                                                          unsigned long long *status, bool iota) {
   constexpr int kTile = kT * kI, kB = 4;
   static_assert(kT >= kRxDigits && kI % kB == 0 && kTile <= 65536, "a thread per digit, whole batches, 16-bit places");
   if (st->skip[pass]) {
@@ -445,8 +445,11 @@ __global__ void __launch_bounds__(kT, 2) rx_sweep(RadixBufs b, RadixState *st, i
   }
   const uint32_t *vin = (c ? b.vals[1] : b.vals[0]) + tbase;
   uint32_t v[kI];
+  if (iota)  // the values are the positions, which nobody has written, until a pass has moved them
+    for (int q = 0; q < pass; ++q) iota = iota && st->skip[q];
 #pragma unroll
-  for (int r = 0; r < kI; ++r) v[r] = first + 32 * r < valid ? vin[first + 32 * r] : 0u;
+  for (int r = 0; r < kI; ++r)
+    v[r] = iota ? (uint32_t)tbase + first + 32 * r : first + 32 * r < valid ? vin[first + 32 * r] : 0u;
   if (d < kRxDigits) {
     uint64_t prefix = 0;  // pairs of digit d in the tiles before this one
     const uint32_t limit = st->spin_limit;
@@ -739,7 +742,7 @@ static vx_status radix_result(char *temp, cudaStream_t s, int *cur) {
 // the low npass bytes of the key (8: the whole key).  The sorted pairs end in
 // buffer st->cur[npass] (0 or 1).
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass,
-                             uint32_t spin_limit) {
+                             uint32_t spin_limit, bool iota) {
   const uint32_t nt = (uint32_t)((n + kSweepTile - 1) / kSweepTile);
   RadixState *st = radix_state_of(temp);
   unsigned long long *bh = (unsigned long long *)(temp + kStateBytes);
@@ -760,7 +763,7 @@ vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s
   // positions take 32 bits below 2^32 pairs
   auto sweep = n >> 32 ? rx_sweep<kSweepThreads, kSweepItems, uint64_t> : rx_sweep<kSweepThreads, kSweepItems, uint32_t>;
   for (int pass = 0; pass < npass; ++pass)  // a skipped pass returns at once and keeps the buffer
-    sweep<<<nt, kSweepThreads, kRxSweepSmem, s>>>(b, st, pass, n, bases, tickets, status);
+    sweep<<<nt, kSweepThreads, kRxSweepSmem, s>>>(b, st, pass, n, bases, tickets, status, iota);
   VX_CUDA_TRY(cudaGetLastError());
   return VX_OK;
 }

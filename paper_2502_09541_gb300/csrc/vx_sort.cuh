@@ -14,9 +14,11 @@ constexpr int kMlpParams = 3 * kMlpHidden + 1;
 uint64_t radix_temp_bytes(uint64_t cap);
 RadixState *radix_state_of(char *temp);
 // spin_limit: polls of one predecessor's look-back word before the pass gives
-// up and sets the error word (0 = the default of 2^20)
+// up and sets the error word (0 = the default of 2^20).  iota: the values are
+// the positions 0 .. n - 1, which need not be in b.vals[0] (when every pass is
+// skipped they are still nowhere)
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass = 8,
-                             uint32_t spin_limit = 0);
+                             uint32_t spin_limit = 0, bool iota = false);
 // after radix_sort_enqueue on s: publishes to a mapped host word the buffer
 // holding the result (low byte), the executed passes (next byte) and whether
 // a look-back wait gave up (bit 16)
