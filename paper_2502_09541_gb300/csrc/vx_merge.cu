@@ -309,6 +309,230 @@ int merge_enqueue(const uint64_t *kin, const uint32_t *vin, const std::vector<ui
   return c;
 }
 
+// ------------------------------------------------------------------ tile merge
+// Merging up to kTileRuns resident runs in one pass over the pairs.  Every
+// stride-th key of every run is a sample; the samples are sorted, and every
+// g-th of them ends a tile.  Between two such samples a run has at most g
+// samples more than the tile's own, so with (g + runs) * stride <= kTilePairs no
+// tile holds more pairs than a block's shared memory takes, whatever the keys
+// (equal keys are told apart by their position in the input, as the merge's
+// order does).  A block loads its tile's pieces of all runs, merges them pairwise
+// in shared memory and writes the tile once: 24 bytes a pair in all, where every
+// pairwise round over the whole partition moves 24.  Bound by the shared-memory
+// rounds.  60M pairs in 64 runs: 2.3 ms of kernels, under the stores, where six
+// pairwise rounds took 4.9 ms and held them up (and 0.42 ms for samples and
+// cuts, 0.29 for the exact cuts before); above 64 runs the samples would be a
+// sixteenth of the pairs and more, and the rounds are kept.
+constexpr uint32_t kTilePairs = 4096, kTileRuns = 64;
+constexpr int kTileThreads = 512, kTileItems = kTilePairs / kTileThreads;
+static_assert(kTileItems == 8, "the padding below spreads chunks of eight");
+
+// shared-memory place of pair x: one pad per eight, so that threads on
+// consecutive chunks of eight use different banks
+__device__ __forceinline__ uint32_t tile_at(uint32_t x) { return x + (x >> 3); }
+constexpr uint32_t kTilePadded = kTilePairs + kTilePairs / 8;
+
+struct TileRuns {
+  uint32_t n_runs, stride;
+  uint64_t off[kTileRuns + 1];     // run r = [off[r], off[r + 1]) of the resident pairs
+  uint32_t sample[kTileRuns + 1];  // its samples' first index
+};
+
+__global__ void tile_sample_kernel(const TileRuns p, const uint64_t *rk, uint64_t *skeys, uint32_t *svals) {
+  const uint32_t ns = p.sample[p.n_runs];
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ns; i += gridDim.x * blockDim.x) {
+    uint32_t a = 0, b = p.n_runs - 1;  // the last run whose samples start at or before i
+    while (a < b) {
+      const uint32_t mid = (a + b + 1) / 2;
+      if (p.sample[mid] <= i) a = mid; else b = mid - 1;
+    }
+    skeys[i] = rk[p.off[a] + (uint64_t)(i - p.sample[a]) * p.stride];
+    svals[i] = i;
+  }
+}
+
+// cut[t * n_runs + r] = pairs of run r before tile t (t <= n_tiles): those
+// before sample t * g of the sorted ones in the order (key, input position)
+__global__ void tile_cuts_kernel(const TileRuns p, const uint64_t *rk, const uint64_t *skeys, const uint32_t *svals,
+                                 uint32_t g, uint32_t n_tiles, uint32_t *cut) {
+  const uint64_t all = (uint64_t)(n_tiles + 1) * p.n_runs;
+  for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < all; j += (uint64_t)gridDim.x * blockDim.x) {
+    // a warp takes neighbouring tiles of one run, whose searches read the same lines nearly to the end
+    const uint32_t t = (uint32_t)(j % (n_tiles + 1)), r = (uint32_t)(j / (n_tiles + 1));
+    const uint64_t i = (uint64_t)t * p.n_runs + r;
+    const uint32_t len = (uint32_t)(p.off[r + 1] - p.off[r]);
+    if (t == 0 || t == n_tiles) {
+      cut[i] = t ? len : 0;
+      continue;
+    }
+    const uint64_t v = skeys[(uint64_t)t * g];
+    const uint32_t at = svals[(uint64_t)t * g];
+    if (at >= p.sample[r] && at < p.sample[r + 1]) {
+      cut[i] = (at - p.sample[r]) * p.stride;
+      continue;
+    }
+    const bool le = at >= p.sample[r + 1];  // a run before the sample's: its equal keys come first
+    const uint64_t *k = rk + p.off[r];
+    uint32_t lo = 0, hi = len;
+    while (lo < hi) {
+      const uint32_t mid = lo + (hi - lo) / 2;
+      if (le ? k[mid] <= v : k[mid] < v) lo = mid + 1; else hi = mid;
+    }
+    cut[i] = lo;
+  }
+}
+
+// rank[t] = pairs before tile t
+__global__ void tile_ranks_kernel(const uint32_t *cut, uint32_t n_runs, uint32_t n_tiles, uint64_t *rank) {
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t <= n_tiles; t += gridDim.x * blockDim.x) {
+    uint64_t s = 0;
+    for (uint32_t r = 0; r < n_runs; ++r) s += cut[(uint64_t)t * n_runs + r];
+    rank[t] = s;
+  }
+}
+
+struct TileSmem {
+  uint64_t k[kTilePadded];
+  uint32_t v[kTilePadded];
+  uint32_t seg[kTileRuns + 1];  // first pair of each non-empty piece
+  uint64_t src[kTileRuns];      // where it is
+  uint32_t nseg, len;
+};
+
+// elements of [a, a + na) among the first d outputs of the stable merge with
+// [a + na, a + na + nb)
+__device__ __forceinline__ uint32_t tile_path(const uint64_t *k, uint32_t a, uint32_t na, uint32_t nb, uint32_t d) {
+  uint32_t lo = d > nb ? d - nb : 0, hi = d < na ? d : na;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) / 2;
+    if (k[tile_at(a + mid)] <= k[tile_at(a + na + d - 1 - mid)]) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// tiles t0 + blockIdx.x; writes the outputs with ranks in [o0, o1)
+__global__ void __launch_bounds__(kTileThreads, 2) tile_merge_kernel(const TileRuns p, const uint64_t *rk,
+                                                                     const uint32_t *rv, const uint32_t *cut,
+                                                                     const uint64_t *rank, uint32_t t0, uint64_t o0,
+                                                                     uint64_t o1, uint64_t *kout, uint32_t *vout) {
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  TileSmem &sm = *reinterpret_cast<TileSmem *>(tile_smem);
+  const uint32_t tile = t0 + blockIdx.x, tid = threadIdx.x;
+  if (tid < 32) {  // the pieces: two runs per lane
+    const uint32_t *c0 = cut + (uint64_t)tile * p.n_runs, *c1 = c0 + p.n_runs;
+    uint32_t len[2], ne[2];
+    uint64_t src[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t r = 2 * tid + q;
+      const uint32_t lo = r < p.n_runs ? c0[r] : 0;
+      len[q] = r < p.n_runs ? c1[r] - lo : 0;
+      src[q] = r < p.n_runs ? p.off[r] + lo : 0;
+      ne[q] = len[q] != 0;
+    }
+    uint32_t x = len[0] + len[1], y = ne[0] + ne[1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t a = __shfl_up_sync(0xffffffffu, x, o), b = __shfl_up_sync(0xffffffffu, y, o);
+      if (tid >= (uint32_t)o) {
+        x += a;
+        y += b;
+      }
+    }
+    uint32_t at = x - len[0] - len[1], id = y - ne[0] - ne[1];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (len[q]) {
+        sm.seg[id] = at;
+        sm.src[id] = src[q];
+        ++id;
+        at += len[q];
+      }
+    if (tid == 31) {
+      sm.seg[y] = x;
+      sm.nseg = y;
+      sm.len = x;
+    }
+  }
+  __syncthreads();
+  uint32_t nseg = sm.nseg;
+  const uint32_t L = sm.len;
+  for (uint32_t x = tid; x < L; x += kTileThreads) {
+    uint32_t a = 0, b = nseg - 1;
+    while (a < b) {
+      const uint32_t mid = (a + b + 1) / 2;
+      if (sm.seg[mid] <= x) a = mid; else b = mid - 1;
+    }
+    const uint64_t i = sm.src[a] + (x - sm.seg[a]);
+    sm.k[tile_at(x)] = rk[i];
+    sm.v[tile_at(x)] = rv[i];
+  }
+  __syncthreads();
+  const uint32_t u0 = tid * kTileItems, u1 = u0 + kTileItems < L ? u0 + kTileItems : L;
+  while (nseg > 1) {
+    uint64_t ok[kTileItems];
+    uint32_t ov[kTileItems];
+    if (u0 < L) {
+      const uint32_t npairs = (nseg + 1) / 2;
+      uint32_t q = 0, b = npairs - 1;  // the pair of pieces that output u0 belongs to
+      while (q < b) {
+        const uint32_t mid = (q + b + 1) / 2;
+        if (sm.seg[2 * mid] <= u0) q = mid; else b = mid - 1;
+      }
+      uint32_t base = sm.seg[2 * q], amid = sm.seg[2 * q + 1], end = 2 * q + 2 <= nseg ? sm.seg[2 * q + 2] : amid;
+      const uint32_t i0 = tile_path(sm.k, base, amid - base, end - amid, u0 - base);
+      uint32_t ia = base + i0, ib = amid + (u0 - base - i0);
+      uint64_t ka = ia < amid ? sm.k[tile_at(ia)] : 0, kb = ib < end ? sm.k[tile_at(ib)] : 0;
+#pragma unroll
+      for (int e = 0; e < kTileItems; ++e) {
+        if (u0 + e < u1) {
+          if (u0 + e == end) {  // the next pair starts
+            ++q;
+            amid = sm.seg[2 * q + 1];
+            ia = end;
+            ib = amid;
+            end = 2 * q + 2 <= nseg ? sm.seg[2 * q + 2] : amid;
+            ka = sm.k[tile_at(ia)];
+            kb = ib < end ? sm.k[tile_at(ib)] : 0;
+          }
+          const bool take_a = ib >= end || (ia < amid && ka <= kb);
+          if (take_a) {
+            ok[e] = ka;
+            ov[e] = sm.v[tile_at(ia)];
+            ++ia;
+            if (ia < amid) ka = sm.k[tile_at(ia)];
+          } else {
+            ok[e] = kb;
+            ov[e] = sm.v[tile_at(ib)];
+            ++ib;
+            if (ib < end) kb = sm.k[tile_at(ib)];
+          }
+        }
+      }
+    }
+    __syncthreads();
+    const uint32_t half = (nseg + 1) / 2;
+    const uint32_t start = tid < half ? sm.seg[2 * tid] : 0;
+#pragma unroll
+    for (int e = 0; e < kTileItems; ++e)
+      if (u0 + e < u1) {
+        sm.k[tile_at(u0 + e)] = ok[e];
+        sm.v[tile_at(u0 + e)] = ov[e];
+      }
+    __syncthreads();
+    if (tid < half) sm.seg[tid] = start;
+    if (tid == half) sm.seg[half] = L;
+    nseg = half;
+    __syncthreads();
+  }
+  const uint64_t r0 = rank[tile];
+  for (uint32_t x = tid; x < L; x += kTileThreads)
+    if (r0 + x >= o0 && r0 + x < o1) {
+      kout[r0 + x - o0] = sm.k[tile_at(x)];
+      vout[r0 + x - o0] = sm.v[tile_at(x)];
+    }
+}
+
 // segment boundaries of the non-empty lengths, starting at 0
 std::vector<uint64_t> segments_of(const std::vector<uint64_t> &lens) {
   std::vector<uint64_t> seg{0};
@@ -569,7 +793,8 @@ struct MergePass : ExKernel {
 // merge pass reads the runs' segments in place.  The pairs cross the link once
 // each way, in copies of whole chunks.  60M pairs in 64 runs (720 MB) under 1
 // GiB: 14.2 ms with the keys loaded to find the runs and the pairs again in 64
-// unaligned pieces a partition, 9.3 ms now, of which the merge rounds take 4.9.
+// unaligned pieces a partition, 9.4 ms with pairwise rounds, 8.2 with the tile
+// merge below.
 
 // the sorted chunk in buffer 0, wherever its radix sort left it
 __global__ void rx_home_kernel(RadixBufs b, const RadixState *st, uint64_t n) {
@@ -674,6 +899,47 @@ struct ResidentMergePass : MergePass {
   }
 };
 
+// merge pass over tiles: partition p is the outputs [p n / P, (p + 1) n / P)
+struct TileMergePass : ExKernel {
+  vx_ctx *ctx;
+  TileRuns runs;
+  const uint64_t *rk;
+  const uint32_t *rv;
+  const uint32_t *d_cut;
+  const uint64_t *d_rank;
+  std::vector<uint64_t> rank;  // n_tiles + 1
+  uint64_t n, P, cap;
+  uint64_t *out_keys;
+  uint32_t *out_vals;
+  int S;
+  uint64_t size() override { return P; }
+  int n_slots() override { return S; }
+  int max_in_flight() override { return S; }
+  uint64_t kb() const { return (8 * cap + 255) & ~255ull; }
+  uint64_t slot_bytes() override { return kb() + ((4 * cap + 255) & ~255ull); }
+  uint64_t at(uint64_t p) const { return p * n / P; }
+  void inputs(uint64_t, char *, std::vector<CopyOp> &) override {}
+  vx_status kernel(char *slot, uint64_t p, cudaStream_t s) override {
+    const uint64_t o0 = at(p), o1 = at(p + 1);
+    if (o0 == o1) return VX_OK;
+    // the tiles that hold outputs o0 .. o1 - 1
+    const uint32_t t0 = (uint32_t)(std::upper_bound(rank.begin(), rank.end(), o0) - rank.begin()) - 1;
+    const uint32_t t1 = (uint32_t)(std::lower_bound(rank.begin(), rank.end(), o1) - rank.begin());
+    tile_merge_kernel<<<t1 - t0, kTileThreads, sizeof(TileSmem), s>>>(runs, rk, rv, d_cut, d_rank, t0, o0, o1,
+                                                                      (uint64_t *)slot, (uint32_t *)(slot + kb()));
+    VX_CUDA_TRY(cudaGetLastError());
+    return VX_OK;
+  }
+  bool has_outputs() override { return true; }
+  vx_status outputs(uint64_t p, char *slot, std::vector<CopyOp> &d2h) override {
+    const uint64_t o0 = at(p), m = at(p + 1) - o0;
+    if (!m) return VX_OK;
+    d2h.push_back({slot, out_keys + o0, 8 * m});
+    d2h.push_back({slot + kb(), out_vals + o0, 4 * m});
+    return VX_OK;
+  }
+};
+
 // exact cuts of runs (keys: device-visible address of the runs) at the given
 // ranks; fences: device, run r's at fence_start[r]
 vx_status exact_cuts(vx_ctx *ctx, const uint64_t *keys, const std::vector<uint64_t> &run_off,
@@ -725,6 +991,99 @@ bool clearly_unsorted(const uint64_t *keys, uint64_t n) {
     desc += keys[i] < keys[i - 1];
   }
   return n > 16 * kMaxRuns && desc * 16 >= ns;
+}
+
+// The merge of 2 to kTileRuns resident runs by tiles into P equal partitions;
+// *done = false: too many runs, or no room for the samples and cuts (then the
+// pairwise rounds take over).
+vx_status tile_merge(vx_ctx *ctx, const uint64_t *rk, const uint32_t *rv, uint64_t n,
+                     const std::vector<uint64_t> &run_off, uint64_t P, uint64_t *out_keys, uint32_t *out_vals,
+                     vx_sort_stats &ss, bool *done) {
+  *done = false;
+  const uint32_t N = (uint32_t)run_off.size() - 1;
+  if (N < 2 || N > kTileRuns || n >> 32) return VX_OK;
+  const double t0 = now_ms();
+  TileRuns runs{};
+  runs.n_runs = N;
+  runs.stride = 256;
+  while (2 * N * runs.stride > kTilePairs) runs.stride /= 2;
+  const uint32_t g = kTilePairs / runs.stride - N;
+  for (uint32_t r = 0; r < N; ++r) {
+    runs.off[r] = run_off[r];
+    runs.sample[r + 1] = runs.sample[r] + (uint32_t)((run_off[r + 1] - run_off[r] + runs.stride - 1) / runs.stride);
+  }
+  runs.off[N] = n;
+  const uint32_t ns = runs.sample[N], n_tiles = (ns + g - 1) / g;
+  cudaStream_t s = ctx->s_compute;
+  DevBuf keep, tmp;
+  keep.arena = tmp.arena = &ctx->arena;
+  const uint64_t rb = (8ull * (n_tiles + 1) + 255) & ~255ull;
+  keep.p = ctx->arena.alloc(rb + 4ull * (n_tiles + 1) * N);
+  const uint64_t skb = (8ull * ns + 255) & ~255ull, svb = (4ull * ns + 255) & ~255ull;
+  tmp.p = keep.p ? ctx->arena.alloc(2 * skb + 2 * svb + radix_temp_bytes(ns)) : nullptr;
+  if (!tmp.p) return VX_OK;
+  uint64_t *d_rank = keep.as<uint64_t>();
+  uint32_t *d_cut = (uint32_t *)(keep.as<char>() + rb);
+  RadixBufs b;
+  b.keys[0] = tmp.as<uint64_t>();
+  b.keys[1] = (uint64_t *)(tmp.as<char>() + skb);
+  b.vals[0] = (uint32_t *)(tmp.as<char>() + 2 * skb);
+  b.vals[1] = (uint32_t *)(tmp.as<char>() + 2 * skb + svb);
+  char *temp = tmp.as<char>() + 2 * skb + 2 * svb;
+  auto grid = [&](uint64_t items) {
+    return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((items + 255) / 256, (uint64_t)ctx->num_sms * 8));
+  };
+  tile_sample_kernel<<<grid(ns), 256, 0, s>>>(runs, rk, b.keys[0], b.vals[0]);
+  VX_TRY(radix_sort_enqueue(b, ns, temp, s, ctx->num_sms, 8, ctx->cfg.lookback_spin_limit));
+  rx_home_kernel<<<grid(ns), 256, 0, s>>>(b, radix_state_of(temp), ns);
+  VX_TRY(radix_publish_enqueue(temp, ctx->d_scalars + 63, s));
+  tile_cuts_kernel<<<grid((uint64_t)(n_tiles + 1) * N), 256, 0, s>>>(runs, rk, b.keys[0], b.vals[0], g, n_tiles, d_cut);
+  tile_ranks_kernel<<<grid(n_tiles + 1), 256, 0, s>>>(d_cut, N, n_tiles, d_rank);
+  VX_CUDA_TRY(cudaGetLastError());
+  TileMergePass mp;
+  mp.rank.resize(n_tiles + 1);
+  VX_CUDA_TRY(cudaMemcpyAsync(mp.rank.data(), d_rank, 8ull * (n_tiles + 1), cudaMemcpyDeviceToHost, s));
+  VX_CUDA_TRY(cudaStreamSynchronize(s));
+  if (((volatile uint64_t *)ctx->h_scalars)[63] >> 16 & 1) {
+    set_error("radix sort of the merge's samples: a look-back wait gave up");
+    return VX_E_TIMEOUT;
+  }
+  tmp.release();
+  ss.ms_sample += now_ms() - t0;
+  const double tq = now_ms();
+  mp.ctx = ctx;
+  mp.runs = runs;
+  mp.rk = rk;
+  mp.rv = rv;
+  mp.d_cut = d_cut;
+  mp.d_rank = d_rank;
+  mp.n = n;
+  mp.P = P;
+  mp.cap = (n + P - 1) / P;
+  mp.out_keys = out_keys;
+  mp.out_vals = out_vals;
+  mp.S = (int)std::min<uint64_t>(kMaxSortSlots, ctx->arena.largest_free() / ((mp.slot_bytes() + 255) & ~255ull));
+  if (mp.S < 2) return VX_OK;
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(tile_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
+  });
+  VX_CUDA_TRY(attr);
+  ExecStats es;
+  VX_TRY(run_pipeline(ctx, mp, &es));
+  ss.bytes_d2h += es.bytes_d2h;
+  ss.kernel_launches += es.kernel_launches + 15;
+  ss.ms_merge_kernel += es.ms_kernel;
+  ss.merge_pass_pairs += n;
+  ss.slot_pairs = mp.cap;
+  ss.ms_sort += now_ms() - tq;
+  ss.n_partitions = (uint32_t)P;
+  ss.max_partition = (n + P - 1) / P;
+  ss.min_partition = n / P;
+  ss.imbalance = (double)ss.max_partition / ((double)n / P);
+  *done = true;
+  return VX_OK;
 }
 
 // The merge plan with resident pairs; *done = false: they do not fit.
@@ -826,6 +1185,8 @@ vx_status resident_merge_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t 
   const uint32_t N = (uint32_t)run_off.size() - 1;
   ss.n_runs = N;
   ss.ms_partition += now_ms() - t0;
+  VX_TRY(tile_merge(ctx, rk, rv, n, run_off, P, out_keys, out_vals, ss, done));
+  if (*done) return VX_OK;
 
   const double ts = now_ms();
   std::vector<uint64_t> ranks, inner;

@@ -82,3 +82,26 @@ def test_runs_mode_and_partitions():
 def test_budget_too_small_goes_through_host_memory():
     n = 3_000_017
     assert _sort(G.sort_input(n, "runs", seed=5)[0], 40)["bytes_h2d"] > 12 * n
+
+
+@pytest.mark.parametrize("n_runs", [2, 5, 8, 9, 33, 63, 64, 65])
+@pytest.mark.parametrize("kind", ["random", "equal", "disjoint", "backward", "few", "lopsided"])
+def test_tiles(n_runs, kind):
+    """Up to 64 runs merge by tiles of at most 4,096 pairs between sorted samples."""
+    n = 1_200_007
+    r = np.random.default_rng(n_runs)
+    cuts = [n * i // n_runs for i in range(n_runs)]
+    if kind == "lopsided":
+        cuts = sorted({0, *(int(x) for x in (r.random(n_runs - 1) ** 4 * n))})
+    k = r.integers(0, 2**64 - 1, n, dtype=np.uint64)
+    if kind == "equal":
+        k[:] = 11
+    elif kind == "few":
+        k %= np.uint64(7)
+    elif kind in ("disjoint", "backward"):
+        for i, (a, b) in enumerate(zip(cuts, cuts[1:] + [n])):
+            k[a:b] = k[a:b] % np.uint64(1000) + np.uint64(1000 * (i if kind == "disjoint" else n_runs - i))
+    for a, b in zip(cuts, cuts[1:] + [n]):
+        k[a:b].sort()
+    st = _sort(k, n_partitions=7)
+    assert st["natural_runs"] == 1 and st["n_partitions"] == 7
