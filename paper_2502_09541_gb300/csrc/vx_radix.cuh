@@ -39,11 +39,13 @@ struct RadixBufs {
 
 // per-pass device state: cur[0..8], skip[0..7], an error word (a look-back
 // wait that gave up), the polls a look-back makes of one predecessor word
-// before giving up, totals[256], base[257]
+// before giving up, a prefix sort's groups left to repair and whether it has to
+// be done again in full, totals[256], base[257]
 struct RadixState {
   int32_t cur[12];
   int32_t skip[12];
   uint32_t err, spin_limit;
+  uint32_t n_fix, redo;
   uint64_t totals[kRxDigits];
   uint64_t base[kRxDigits + 1];
 };

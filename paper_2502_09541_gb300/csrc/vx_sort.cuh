@@ -19,9 +19,16 @@ RadixState *radix_state_of(char *temp);
 // skipped they are still nowhere)
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass = 8,
                              uint32_t spin_limit = 0, bool iota = false);
+// The same for n < 2^32 pairs whose keys nearly all differ in their upper bytes:
+// passes over the key bytes first .. 7 only, then the few groups of pairs that
+// agree in all of those are put in order where they are.  If a group is large
+// or there are many, bit 17 of the published word says that the pairs (a
+// stable rearrangement of the input) have to be sorted in full.
+vx_status radix_prefix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int first,
+                                    uint32_t spin_limit);
 // after radix_sort_enqueue on s: publishes to a mapped host word the buffer
-// holding the result (low byte), the executed passes (next byte) and whether
-// a look-back wait gave up (bit 16)
+// holding the result (low byte), the executed passes (next byte), whether
+// a look-back wait gave up (bit 16) and the prefix sort's bit 17
 vx_status radix_publish_enqueue(char *temp, uint64_t *host_word, cudaStream_t s, int npass = 8);
 vx_status range_partition_enqueue(RadixBufs b, uint64_t n, const uint64_t *spl, uint32_t P, char *temp,
                                   cudaStream_t s);
