@@ -91,8 +91,9 @@ struct CudaDev {
     }
     VX_TRY(issue_copies(ops, cudaMemcpyHostToDevice, ctx->s_h2d, &st->bytes_h2d, h2d_sm_blocks(ctx)));
     if (tl) VX_CUDA_TRY(cudaEventRecord(sl.ev_h1, ctx->s_h2d));
-    VX_CUDA_TRY(cudaEventRecord(sl.ev_in, ctx->s_h2d));
-    VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_compute, sl.ev_in, 0));
+    cudaEvent_t in = k.loaded_event(it);
+    if (!in) VX_CUDA_TRY(cudaEventRecord(in = sl.ev_in, ctx->s_h2d));
+    VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_compute, in, 0));
     VX_CUDA_TRY(cudaEventRecord(sl.ev_k0, ctx->s_compute));
     VX_TRY(k.kernel(slot(s), it, ctx->s_compute));
     st->kernel_launches += 1;
@@ -301,14 +302,15 @@ vx_status run_pipeline(vx_ctx *ctx, ExKernel &k, ExecStats *st) {
   const uint64_t slot_bytes = (k.slot_bytes() + 255) & ~255ull;
   DevBuf ring;
   ring.arena = &ctx->arena;
-  ring.p = ctx->arena.alloc(slot_bytes * (uint64_t)S);
-  if (!ring.p) {
+  char *own = k.ring();
+  if (!own) ring.p = ctx->arena.alloc(slot_bytes * (uint64_t)S);
+  if (!own && !ring.p) {
     set_error("executor: %d slots of %llu bytes do not fit the arena (%llu of %llu bytes free)", S,
               (unsigned long long)slot_bytes, (unsigned long long)ctx->arena.largest_free(),
               (unsigned long long)ctx->arena.capacity());
     return VX_E_NOMEM;
   }
-  char *base = ring.as<char>();
+  char *base = own ? own : ring.as<char>();
   EventSet es;
   es.s.resize(S);
   for (auto &x : es.s) {
@@ -338,8 +340,9 @@ vx_status run_pipeline(vx_ctx *ctx, ExKernel &k, ExecStats *st) {
       ops.clear();
       k.inputs(it, slot, ops);
       VX_TRY(issue_copies(ops, cudaMemcpyHostToDevice, ctx->s_h2d, &st->bytes_h2d, h2d_sm_blocks(ctx)));
-      VX_CUDA_TRY(cudaEventRecord(sl.ev_in, ctx->s_h2d));
-      VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_compute, sl.ev_in, 0));
+      cudaEvent_t in = k.loaded_event(it);
+      if (!in) VX_CUDA_TRY(cudaEventRecord(in = sl.ev_in, ctx->s_h2d));
+      VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_compute, in, 0));
       VX_TRY(k.kernel(slot, it, ctx->s_compute));
       st->kernel_launches += 1;
       VX_CUDA_TRY(cudaEventRecord(sl.ev_k, ctx->s_compute));

@@ -201,6 +201,12 @@ struct ExKernel {
   // schedule keeps in flight at once (loaded, computing or storing)
   virtual int n_slots() { return 0; }
   virtual int max_in_flight() { return 3; }
+  // the ring, if the operator brings its own (n_slots() of slot_bytes() rounded
+  // up to 256, which outlives the pipeline); null: allocated for the run
+  virtual char *ring() { return nullptr; }
+  // event after the copies of a chunk that were issued before the run (its
+  // inputs() is empty); null: the run issues them
+  virtual cudaEvent_t loaded_event(uint64_t it) { return nullptr; }
 };
 
 struct ExecStats {

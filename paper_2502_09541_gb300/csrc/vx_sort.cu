@@ -974,7 +974,7 @@ vx_status splitters_from_sample(vx_ctx *ctx, int32_t kind, const uint64_t *sorte
 // samples m keys of a mapped column and sorts them on the device; m shrinks to
 // what the free arena holds
 vx_status sample_and_sort(vx_ctx *ctx, const uint64_t *dev_keys, uint64_t n, uint64_t &m, uint64_t seed,
-                          DevBuf &sorted_out, uint64_t **sorted_ptr) {
+                          DevBuf &sorted_out, uint64_t **sorted_ptr, const std::function<vx_status()> &sampled) {
   cudaStream_t s = ctx->s_compute;
   const uint64_t freeb = ctx->arena.largest_free();
   const uint64_t m_fit = freeb > (64u << 10) ? (freeb - (64u << 10)) / 25 : 0;
@@ -1000,6 +1000,7 @@ vx_status sample_and_sort(vx_ctx *ctx, const uint64_t *dev_keys, uint64_t n, uin
   char *temp = q + 2 * ((4 * m + 255) & ~255ull);
   sample_keys_kernel<<<ctx->num_sms * 2, 256, 0, s>>>(dev_keys, n, m, seed, b.keys[0], b.vals[0]);
   VX_CUDA_TRY(cudaGetLastError());
+  if (sampled) VX_TRY(sampled());
   VX_TRY(radix_sort_enqueue(b, m, temp, s, ctx->num_sms, 8, ctx->cfg.lookback_spin_limit));
   int cur = 0;
   VX_TRY(radix_result(temp, s, &cur));
@@ -1232,14 +1233,34 @@ struct SortPass : ExKernel {
 // scatters the chunks straight into the partitions' regions and pass 2 sorts
 // each partition where it is (the other buffer in a slot) and stores it: the
 // pairs cross the link once in each direction instead of twice.  67M uniform
-// pairs (805 MB) under 1 GiB: 10.3 ms, 13.7 through host memory; 300M (3.6 GB)
-// under 4.5 GiB: 39 ms, about 62.  Bound by the link one way, then the other,
-// and by the partition sorts (5.0 of the 5.7 ms of pass 2).
+// pairs (805 MB) under 1 GiB: 10.3 ms, 13.7 through host memory (9.05 with the
+// shorter sorts and the early loads below); 300M (3.6 GB) under 4.5 GiB: 37.5
+// ms, about 62.  Bound by the link one way, then the other.
 struct ResidentPlan {
   std::vector<uint64_t> off, cap;  // regions, pairs
   uint64_t pairs = 0;              // all regions
   uint64_t R = 0, jcap = 0;        // pairs per slot of pass 1 and pass 2
   int S1 = 0, S2 = 0;
+  // pass 1's slots, which take what the regions leave of the arena; the first
+  // chunks are loaded into them while the splitters are still being found (the
+  // sample's sort, the model's training), and pass 2's slots follow in their
+  // place.  50M pairs with the MLP partitioner, whose training takes 1.9 ms: 9.7
+  // -> 8.1 ms; 67M with the sample's quantiles 9.3 -> 9.05.
+  vx_ctx *ctx = nullptr;
+  DevBuf ring;
+  std::vector<cudaEvent_t> loaded;  // one per chunk, after its copies
+  uint64_t bytes_loaded = 0;
+  bool drain = false;
+  void release() {
+    if (!ring.p) return;
+    if (ctx->poisoned) ring.arena = nullptr;  // work that never finished may still write there
+    else if (drain) cudaStreamSynchronize(ctx->s_h2d);
+    ring.release();
+  }
+  ~ResidentPlan() {
+    release();
+    for (cudaEvent_t e : loaded) cudaEventDestroy(e);
+  }
 };
 
 struct ResidentPartitionPass : ExKernel {
@@ -1252,14 +1273,20 @@ struct ResidentPartitionPass : ExKernel {
   uint64_t *res_keys;
   uint32_t *res_vals;
   RxRegions *rg;
+  char *base;  // the ring
+  const std::vector<cudaEvent_t> *loaded = nullptr;  // chunks whose copies have been issued
   uint64_t size() override { return (n + R - 1) / R; }
   int n_slots() override { return S; }
+  int max_in_flight() override { return S; }
+  char *ring() override { return base; }
+  cudaEvent_t loaded_event(uint64_t it) override { return loaded && it < loaded->size() ? (*loaded)[it] : nullptr; }
   uint64_t rows(uint64_t it) const { return std::min(R, n - it * R); }
   uint64_t kb() const { return (8 * R + 255) & ~255ull; }
   uint64_t vb() const { return (4 * R + 255) & ~255ull; }
   static uint64_t bytes(uint64_t R) { return (8 * R + 255) / 256 * 256 + (4 * R + 255) / 256 * 256 + radix_temp_bytes(R); }
   uint64_t slot_bytes() override { return bytes(R); }
   void inputs(uint64_t it, char *slot, std::vector<CopyOp> &h2d) override {
+    if (loaded_event(it)) return;
     h2d.push_back({keys + it * R, slot, 8 * rows(it)});
     h2d.push_back({vals + it * R, slot + kb(), 4 * rows(it)});
   }
@@ -1350,22 +1377,83 @@ bool single_key_partition(const std::vector<uint64_t> &spl, uint32_t p) {
   return p < spl.size() ? (spl[p] > lo && spl[p] - lo == 1) : lo == UINT64_MAX;
 }
 
-// Partitions requested so that the regions, and two slots of pass 2 beside
-// them, fit `avail` bytes with room for uneven partitions; 0: they do not fit.
-uint32_t resident_partitions(uint64_t n, uint64_t avail, double headroom) {
-  const double left = (double)avail - 12.0 * 1.03 * (double)n - (1 << 20);
-  if (left <= 0) return 0;
-  const double jcap = left / (2 * 12.6);
+// Bytes of the arena that P regions (with their headroom, see resident_layout)
+// leave to the slots; m sampled keys
+uint64_t resident_left(uint64_t n, uint64_t m, uint32_t P, uint64_t avail) {
+  const double pairs = 1.002 * (double)n +
+                       P * (6.0 * std::sqrt((double)m / P + 1.0) * (double)n / (double)m + kRxTile + 128.0);
+  const double left = (double)avail - 12.0 * pairs - (1 << 20);
+  return left > 0 ? (uint64_t)left : 0;
+}
+
+// Partitions requested so that two slots of pass 2 fit what the regions leave,
+// with room for uneven partitions; 0: they do not fit.
+uint32_t resident_partitions(uint64_t n, uint64_t m, uint64_t avail, double headroom) {
   // at most 12M pairs a job, so that the stores start early
-  const double P = std::max(std::ceil(headroom * (double)n / jcap), std::ceil((double)n / 12e6));
-  return P > 64 ? 0u : std::max<uint32_t>((uint32_t)P, 4);
+  double P = std::max(4.0, std::ceil((double)n / 12e6));
+  for (int i = 0; i < 8 && P <= 64; ++i) {
+    const double jcap = (double)resident_left(n, m, (uint32_t)P, avail) / (2 * 12.6);
+    if (jcap < 1) return 0;
+    if (headroom * (double)n / jcap <= P) return (uint32_t)P;
+    P = std::ceil(headroom * (double)n / jcap);
+  }
+  return 0;
+}
+
+// Pass 1's ring: chunks of n / 16 pairs (smaller if S slots of them do not fit),
+// as many slots as fit and are of use.  False: no room.
+bool resident_ring(vx_ctx *ctx, uint64_t n, uint64_t left, int S, ResidentPlan *rp) {
+  auto slot = [](uint64_t R) { return (ResidentPartitionPass::bytes(R) + 255) & ~255ull; };
+  for (rp->R = std::min<uint64_t>(std::max<uint64_t>(n / 16, 1 << 20), kPipelineRows) / kRxTile * kRxTile;
+       rp->R >= (1 << 18); rp->R = rp->R / 2 / kRxTile * kRxTile)
+    if ((uint64_t)S * slot(rp->R) <= left) break;
+  if (rp->R < (1 << 18)) return false;
+  rp->S1 = (int)std::max<uint64_t>(S, std::min<uint64_t>({left / slot(rp->R), (n + rp->R - 1) / rp->R, 12}));
+  rp->ctx = ctx;
+  rp->ring.arena = &ctx->arena;
+  rp->ring.bytes = std::max<uint64_t>(rp->S1 * slot(rp->R), std::min<uint64_t>(left, 2 * 13 * 13000000ull));
+  rp->ring.p = ctx->arena.alloc(rp->ring.bytes);
+  return rp->ring.p != nullptr;
+}
+
+// Loads the first chunks into the ring on the host-to-device stream, behind the
+// work that the compute stream has now.
+vx_status resident_prefetch(const uint64_t *keys, const uint32_t *vals, uint64_t n, ResidentPlan *rp) {
+  vx_ctx *ctx = rp->ctx;
+  cudaEvent_t e;
+  VX_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  struct Free {
+    cudaEvent_t e;
+    ~Free() { cudaEventDestroy(e); }
+  } fr{e};
+  VX_CUDA_TRY(cudaEventRecord(e, ctx->s_compute));
+  VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_h2d, e, 0));
+  ResidentPartitionPass pp;
+  pp.keys = keys;
+  pp.vals = vals;
+  pp.n = n;
+  pp.R = rp->R;
+  std::vector<CopyOp> ops;
+  rp->drain = true;
+  const uint64_t slot = (pp.slot_bytes() + 255) & ~255ull, k = std::min<uint64_t>(pp.size(), rp->S1);
+  for (uint64_t it = 0; it < k; ++it) {
+    ops.clear();
+    pp.inputs(it, rp->ring.as<char>() + it * slot, ops);
+    VX_TRY(issue_copies(ops, cudaMemcpyHostToDevice, ctx->s_h2d, &rp->bytes_loaded, h2d_sm_blocks(ctx)));
+    cudaEvent_t done;
+    VX_CUDA_TRY(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
+    rp->loaded.push_back(done);
+    VX_CUDA_TRY(cudaEventRecord(done, ctx->s_h2d));
+  }
+  return VX_OK;
 }
 
 // Regions from the sample's count in each partition: the estimate plus 0.2 %
 // and six standard deviations (a region that is too small all the same ends the
-// attempt).  False if regions and slots do not fit `avail` bytes.
+// attempt).  False if the regions do not fit `rest` bytes or two slots of pass
+// 2 the ring's.
 bool resident_layout(uint64_t n, uint64_t m, const std::vector<uint64_t> &spl, const std::vector<uint64_t> &srank,
-                     uint64_t avail, int S, ResidentPlan *rp) {
+                     uint64_t rest, ResidentPlan *rp) {
   const uint32_t P = (uint32_t)spl.size() + 1;
   rp->off.resize(P);
   rp->cap.resize(P);
@@ -1380,16 +1468,8 @@ bool resident_layout(uint64_t n, uint64_t m, const std::vector<uint64_t> &spl, c
     if (!single_key_partition(spl, p)) rp->jcap = std::max(rp->jcap, rp->cap[p]);
   }
   rp->jcap = std::max<uint64_t>(rp->jcap, kRxTile);
-  const uint64_t fixed = 12 * rp->pairs + sizeof(RxRegions) + 4096;
-  if (fixed >= avail) return false;
-  const uint64_t left = avail - fixed;
-  rp->S2 = (int)std::min<uint64_t>(kMaxSortSlots, left / (ResidentPartitionPass::bytes(rp->jcap) + 256));
-  if (rp->S2 < 2) return false;
-  rp->S1 = S;
-  for (rp->R = std::min<uint64_t>(std::max<uint64_t>(n / 16, 1 << 20), kPipelineRows) / kRxTile * kRxTile;
-       rp->R >= (1 << 18); rp->R = rp->R / 2 / kRxTile * kRxTile)
-    if ((uint64_t)S * (ResidentPartitionPass::bytes(rp->R) + 256) <= left) return true;
-  return false;
+  rp->S2 = (int)std::min<uint64_t>(kMaxSortSlots, rp->ring.bytes / ((ResidentPartitionPass::bytes(rp->jcap) + 255) & ~255ull));
+  return rp->S2 >= 2 && 12 * rp->pairs + sizeof(RxRegions) + 4096 <= rest;
 }
 
 // How many low key bytes (4, 3 or 0) the sorts may leave to a repair, from the
@@ -1415,7 +1495,7 @@ int prefix_bytes(const uint64_t (&c)[4], uint64_t m, uint64_t n) {
 // (nothing has been written to the output; the caller sorts the other way).
 vx_status resident_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals, uint64_t n, uint64_t *out_keys,
                         uint32_t *out_vals, const uint64_t *d_spl, const std::vector<uint64_t> &spl,
-                        const ResidentPlan &rp, int first, vx_sort_stats &ss, bool *done) {
+                        ResidentPlan &rp, int first, vx_sort_stats &ss, bool *done) {
   const uint32_t P = (uint32_t)spl.size() + 1;
   *done = false;
   DevBuf mem;
@@ -1447,12 +1527,15 @@ vx_status resident_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals,
     pp.res_keys = res_keys;
     pp.res_vals = res_vals;
     pp.rg = rg;
+    pp.base = rp.ring.as<char>();
+    pp.loaded = &rp.loaded;
     ExecStats es;
     VX_TRY(run_pipeline(ctx, pp, &es));
     VX_CUDA_TRY(cudaMemcpyAsync(h.get(), rg, sizeof(RxRegions), cudaMemcpyDeviceToHost, s));
     VX_CUDA_TRY(cudaStreamSynchronize(s));
     ss.bytes_h2d += es.bytes_h2d;
     ss.kernel_launches += es.kernel_launches * 4;  // upsweep, row scan, placement, scatter
+    rp.release();  // pass 2's slots take the ring's place
   }
   ss.ms_partition += now_ms() - t0;
   if (h->full) return VX_OK;
@@ -1563,8 +1646,25 @@ static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *v
     return VX_E_NOMEM;
   }
   uint64_t *d_spl = splbuf.as<uint64_t>();
-  const uint64_t pass_avail = ctx->arena.largest_free();  // for the passes, once the sample is gone
-  VX_TRY(sample_and_sort(ctx, dev_keys, n, m, o.seed + (uint64_t)depth * 7919, sbuf, &sorted));
+  // resident partitions, where the caller has not bounded the slots or the
+  // regions (a smooth model's partitions are less even than the sample's): the
+  // ring comes first in the arena, so that what is left is in one piece once the
+  // sample is gone
+  const uint32_t P_out = P;
+  uint32_t P_in = 0;
+  ResidentPlan rp;
+  uint64_t rest = 0;
+  if (may_reside && depth == 0 && !o.max_slot_pairs && !o.region_slack_pct) {
+    const uint64_t avail = ctx->arena.largest_free();
+    P_in = resident_partitions(n, m, avail, o.partitioner == VX_PART_LEARNED_MLP ? 1.4 : 1.1);
+    if (P_in && o.n_partitions > 1) P_in = (uint32_t)o.n_partitions;
+    if (P_in && !resident_ring(ctx, n, resident_left(n, m, P_in, avail), S, &rp)) P_in = 0;
+    rest = ctx->arena.largest_free();
+  }
+  VX_TRY(sample_and_sort(ctx, dev_keys, n, m, o.seed + (uint64_t)depth * 7919, sbuf, &sorted, [&]() -> vx_status {
+    return P_in ? resident_prefetch(keys, vals, n, &rp) : VX_OK;
+  }));
+  ss.bytes_h2d += rp.bytes_loaded;
   double ms_train = 0;
   uint32_t n_spl = 0;
   std::vector<uint64_t> spl, srank;
@@ -1594,32 +1694,22 @@ static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *v
     VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
     return VX_OK;
   };
-  // resident partitions, where the caller has not bounded the slots or the
-  // regions: a smooth model's partitions are less even than the sample's
-  const uint32_t P_out = P;
-  ResidentPlan rp;
   int first = 0;  // key bytes that the partitions' sorts may leave to a repair
   bool reside = false;
-  if (may_reside && depth == 0 && !o.max_slot_pairs && !o.region_slack_pct) {
-    uint32_t P_in = resident_partitions(n, pass_avail, o.partitioner == VX_PART_LEARNED_MLP ? 1.4 : 1.1);
-    if (P_in && o.n_partitions > 1) P_in = (uint32_t)o.n_partitions;
-    if (P_in) {
-      pbuf.p = ctx->arena.alloc(sizeof prefix);
-      if (pbuf.p) {
-        VX_CUDA_TRY(cudaMemsetAsync(pbuf.p, 0, sizeof prefix, ctx->s_compute));
-        sample_prefix_kernel<<<ctx->num_sms * 4, 256, 0, ctx->s_compute>>>(sorted, m, pbuf.as<unsigned long long>());
-        VX_CUDA_TRY(cudaGetLastError());
-      }
-      VX_TRY(cut(P_in));
-      reside = resident_layout(n, m, spl, srank, pass_avail, S, &rp);
-      if (pbuf.p) first = prefix_bytes(prefix, m, n);
-      pbuf.release();
+  if (P_in) {
+    pbuf.p = ctx->arena.alloc(sizeof prefix);
+    if (pbuf.p) {
+      VX_CUDA_TRY(cudaMemsetAsync(pbuf.p, 0, sizeof prefix, ctx->s_compute));
+      sample_prefix_kernel<<<ctx->num_sms * 4, 256, 0, ctx->s_compute>>>(sorted, m, pbuf.as<unsigned long long>());
+      VX_CUDA_TRY(cudaGetLastError());
     }
-    if (!reside && P_in != P_out) n_spl = 0, spl.clear(), P_in = 0;
-    if (!P_in) VX_TRY(cut(P_out));
-  } else {
-    VX_TRY(cut(P_out));
+    VX_TRY(cut(P_in));
+    reside = resident_layout(n, m, spl, srank, rest, &rp);
+    if (pbuf.p) first = prefix_bytes(prefix, m, n);
+    pbuf.release();
+    if (!reside) rp.release();
   }
+  if (!reside && P_in != P_out) VX_TRY(cut(P_out));
   sbuf.release();
   ss.ms_sample += now_ms() - ts - ms_train;
   ss.ms_train += ms_train;
@@ -1628,6 +1718,7 @@ static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *v
     bool done = false;
     VX_TRY(resident_sort(ctx, keys, vals, n, out_keys, out_vals, d_spl, spl, rp, first, ss, &done));
     if (done) return VX_OK;
+    rp.release();
     splbuf.release();
     return sort_pairs(ctx, keys, vals, dev_keys, n, out_keys, out_vals, o, ss, depth, false);
   }

@@ -60,8 +60,11 @@ vx_status merge_sort_plan(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
                           uint64_t n, uint64_t *out_keys, uint32_t *out_vals, const vx_sort_opts &o,
                           vx_sort_stats &ss);
 
+// sampled: called once the sampling kernel (which reads host memory over the
+// link) is enqueued, before the sort
 vx_status sample_and_sort(vx_ctx *ctx, const uint64_t *dev_keys, uint64_t n, uint64_t &m, uint64_t seed,
-                          DevBuf &sorted_out, uint64_t **sorted_ptr);
+                          DevBuf &sorted_out, uint64_t **sorted_ptr,
+                          const std::function<vx_status()> &sampled = nullptr);
 // splitters for P requested partitions from a sorted device sample with
 // partitioner `kind`, then heavy-key isolation; *n_spl receives their count
 vx_status splitters_from_sample(vx_ctx *ctx, int32_t kind, const uint64_t *sorted, uint64_t m, uint32_t P,
