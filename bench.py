@@ -582,7 +582,7 @@ def run_sort_extra(vx, G, args):
         if st["ms_sort_kernel"] > 0:
             hbm_peak, peak_kind = measured_peaks()
             ach = 24 * st["radix_pass_pairs"] / (st["ms_sort_kernel"] * 1e6)
-            out["radix_roofline"] = {"kernel": "rx_downsweep (one-sweep LSD pass)", "bound": "hbm", "unit": "GB/s",
+            out["radix_roofline"] = {"kernel": "rx_sweep (one-sweep LSD pass)", "bound": "hbm", "unit": "GB/s",
                                      "achieved": round(ach, 1), "peak": hbm_peak, "frac": round(ach / hbm_peak, 4),
                                      "peak_kind": peak_kind, "pass_pairs": int(st["radix_pass_pairs"]),
                                      "ms_sort_kernel": round(st["ms_sort_kernel"], 1)}

@@ -316,22 +316,6 @@ __global__ void __launch_bounds__(kRxThreads, 2) rx_range_scatter(RadixBufs b, c
   }
 }
 
-// One LSD pass: a stable scatter of the pairs by one key byte.  The tile is
-// the block's ticket; its digits' positions come from the one-read histogram
-// (bases) plus a look-back over the status words of the tiles before it.
-//   rank: a warp owns kI * 32 consecutive pairs.  The lanes of a round that
-// share a digit find one another (match_any), their first lane adds them to the
-// warp's counter of the digit and hands the count before them to the others;
-// the rounds' matches and shared-memory atomics are issued back to back, so
-// that the warp waits for one round trip per kB rounds and not for each.
-//   place: keys are regrouped by digit in shared memory while the tiles before
-// publish, then written as runs of consecutive positions; the values follow
-// through the same shared memory.  Holding only one of the two at a time lets
-// 28 warps share an SM, which the latencies here need.
-// Bound by shared-memory wavefronts, barriers and issue rather than by HBM: 24
-// bytes a pair and pass at 3.25 TB/s (0.48 of the measured copy bandwidth, 40M
-// pairs); 1.67 TB/s before, when every round waited for its match_any and its
-// counter, and keys and values together left 16 warps an SM.
 // Lanes of the warp with the same 8-bit digit, from one vote per bit
 // (match_any takes a step per distinct value, about 30 of them for random
 // digits: 0.98 against 0.74 ms for the eight passes over 9.6M random pairs,
@@ -347,6 +331,22 @@ __device__ __forceinline__ uint32_t same_digit(uint32_t d) {
   return peers;
 }
 
+// One LSD pass: a stable scatter of the pairs by one key byte.  The tile is
+// the block's ticket; its digits' positions come from the one-read histogram
+// (bases) plus a look-back over the status words of the tiles before it.
+//   rank: a warp owns kI * 32 consecutive pairs.  The lanes of a round that
+// share a digit find one another (same_digit), their first lane adds them to the
+// warp's counter of the digit and hands the count before them to the others;
+// the rounds' matches and shared-memory atomics are issued back to back, so
+// that the warp waits for one round trip per kB rounds and not for each.
+//   place: keys are regrouped by digit in shared memory while the tiles before
+// publish, then written as runs of consecutive positions; the values follow
+// through the same shared memory.  Holding only one of the two at a time lets
+// 28 warps share an SM, which the latencies here need.
+// Bound by shared-memory wavefronts, barriers and issue rather than by HBM: 24
+// bytes a pair and pass at 3.25 TB/s (0.48 of the measured copy bandwidth, 40M
+// pairs); 1.67 TB/s before, when every round waited for its match_any and its
+// counter, and keys and values together left 16 warps an SM.
 template <int kT, int kI, class Off>
 struct RxSweepSmem {
   uint64_t k[kT * kI];                 // the keys by digit, then the values
@@ -1808,7 +1808,7 @@ static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *v
     VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
     ss.bytes_h2d += es.bytes_h2d;
     ss.bytes_d2h += es.bytes_d2h;
-    ss.kernel_launches += es.kernel_launches * 4;  // upsweep, row scan, totals, downsweep
+    ss.kernel_launches += es.kernel_launches * 4;  // upsweep, row scan, totals, scatter
   }
   ss.ms_partition += now_ms() - tp;
 
