@@ -517,19 +517,52 @@ constexpr size_t kRxScatterSmem = sizeof(RxScatterSmem);
 
 // 14 warps a block, two blocks an SM, 72 registers a thread: eight passes over
 // 9.6M / 40M random pairs take 0.666 / 2.36 ms; 512 x 2 (64 registers, spilling
-// more) 0.683 / 2.40, 384 x 3 0.750 / 2.59, 256 x 4 0.723 / 2.48
-constexpr int kSweepThreads = 448, kSweepItems = 16;
-constexpr uint32_t kSweepTile = kSweepThreads * kSweepItems;
-constexpr size_t kRxSweepSmem = sizeof(RxSweepSmem<kSweepThreads, kSweepItems, uint64_t>);
+// more) 0.683 / 2.40, 384 x 3 0.750 / 2.59, 256 x 4 0.723 / 2.48.  16 pairs a
+// thread, or 8 while that leaves no SM a second block: a small sort's time is a
+// tile's chain of steps (8 passes over 100K / 500K pairs take 0.103 / 0.123 ms
+// with 8, 0.119 / 0.142 with 16; over 1M 0.160 and 0.158).
+constexpr int kSweepThreads = 448;
+constexpr uint32_t kSweepTile = kSweepThreads * 16, kSweepSmallTile = kSweepThreads * 8;
+constexpr uint32_t kSweepSmallTiles = 160;  // small tiles a sort may have, by num_sms or at most so many
+
+static bool sweep_small(uint64_t n, int num_sms) {
+  return n <= (uint64_t)kSweepSmallTile * std::min<uint32_t>(num_sms, kSweepSmallTiles);
+}
+static uint32_t sweep_tiles(uint64_t n, int num_sms) {
+  const uint32_t t = sweep_small(n, num_sms) ? kSweepSmallTile : kSweepTile;
+  return (uint32_t)((n + t - 1) / t);
+}
+
+template <int kI, class Off>
+static vx_status launch_sweep(RadixBufs b, RadixState *st, int pass, uint64_t n, const uint64_t *bases,
+                              unsigned int *tickets, unsigned long long *status, bool iota, uint32_t tiles,
+                              cudaStream_t s) {
+  constexpr size_t smem = sizeof(RxSweepSmem<kSweepThreads, kI, Off>);
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(rx_sweep<kSweepThreads, kI, Off>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem);
+  });
+  VX_CUDA_TRY(attr);
+  rx_sweep<kSweepThreads, kI, Off><<<tiles, kSweepThreads, smem, s>>>(b, st, pass, n, bases, tickets, status, iota);
+  return VX_OK;
+}
+
+// one pass; positions take 32 bits below 2^32 pairs
+static vx_status enqueue_sweep(RadixBufs b, RadixState *st, int pass, uint64_t n, const uint64_t *bases,
+                               unsigned int *tickets, unsigned long long *status, bool iota, int num_sms,
+                               cudaStream_t s) {
+  const uint32_t nt = sweep_tiles(n, num_sms);
+  if (sweep_small(n, num_sms)) return launch_sweep<8, uint32_t>(b, st, pass, n, bases, tickets, status, iota, nt, s);
+  if (n >> 32) return launch_sweep<16, uint64_t>(b, st, pass, n, bases, tickets, status, iota, nt, s);
+  return launch_sweep<16, uint32_t>(b, st, pass, n, bases, tickets, status, iota, nt, s);
+}
 
 // the scatters' shared memory is above the 48 KB default: raise the limit once
 static vx_status rx_scatter_attr() {
   static bool done = false;
   if (!done) {
-    VX_CUDA_TRY(cudaFuncSetAttribute(rx_sweep<kSweepThreads, kSweepItems, uint32_t>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRxSweepSmem));
-    VX_CUDA_TRY(cudaFuncSetAttribute(rx_sweep<kSweepThreads, kSweepItems, uint64_t>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRxSweepSmem));
     VX_CUDA_TRY(cudaFuncSetAttribute(rx_range_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kRxScatterSmem));
     done = true;
@@ -808,7 +841,9 @@ constexpr uint64_t kBasesBytes = 8ull * kRxDigits * 8;
 constexpr uint64_t kTicketBytes = 256;
 
 uint64_t radix_temp_bytes(uint64_t cap) {
-  const uint64_t nt = std::max<uint32_t>(ntiles_of(cap), 1);
+  // the sweep's tiles hold more, but for a small sort's
+  const uint64_t nt = std::max<uint64_t>(
+      {ntiles_of(cap), 1, std::min<uint64_t>((cap + kSweepSmallTile - 1) / kSweepSmallTile, kSweepSmallTiles)});
   return kStateBytes + kByteHistBytes + kBasesBytes + kTicketBytes + (uint64_t)kRxDigits * nt * 8 + 256;
 }
 
@@ -833,7 +868,7 @@ static vx_status radix_result(char *temp, cudaStream_t s, int *cur) {
 // buffer st->cur[npass] (0 or 1).
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass,
                              uint32_t spin_limit, bool iota) {
-  const uint32_t nt = (uint32_t)((n + kSweepTile - 1) / kSweepTile);
+  const uint32_t nt = sweep_tiles(n, num_sms);
   RadixState *st = radix_state_of(temp);
   unsigned long long *bh = (unsigned long long *)(temp + kStateBytes);
   uint64_t *bases = (uint64_t *)(temp + kStateBytes + kByteHistBytes);
@@ -850,10 +885,8 @@ vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s
   auto hist = npass == 1 ? rx_byte_hist<1> : npass == 2 ? rx_byte_hist<2> : npass == 3 ? rx_byte_hist<3> : rx_byte_hist<8>;
   hist<<<g, kRxThreads, 0, s>>>(b.keys[0], n, bh);
   rx_init<<<npass, kRxDigits, 0, s>>>(st, bh, bases, n, spin_limit ? spin_limit : kRxSpinLimit, 0);
-  // positions take 32 bits below 2^32 pairs
-  auto sweep = n >> 32 ? rx_sweep<kSweepThreads, kSweepItems, uint64_t> : rx_sweep<kSweepThreads, kSweepItems, uint32_t>;
   for (int pass = 0; pass < npass; ++pass)  // a skipped pass returns at once and keeps the buffer
-    sweep<<<nt, kSweepThreads, kRxSweepSmem, s>>>(b, st, pass, n, bases, tickets, status, iota);
+    VX_TRY(enqueue_sweep(b, st, pass, n, bases, tickets, status, iota, num_sms, s));
   VX_CUDA_TRY(cudaGetLastError());
   return VX_OK;
 }
@@ -862,7 +895,7 @@ vx_status radix_prefix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStr
                                     uint32_t spin_limit) {
   if (n < 2 || n >> 32 || (first != 3 && first != 4))
     return radix_sort_enqueue(b, n, temp, s, num_sms, 8, spin_limit);
-  const uint32_t nt = (uint32_t)((n + kSweepTile - 1) / kSweepTile);
+  const uint32_t nt = sweep_tiles(n, num_sms);
   RadixState *st = radix_state_of(temp);
   unsigned long long *bh = (unsigned long long *)(temp + kStateBytes);
   uint64_t *bases = (uint64_t *)(temp + kStateBytes + kByteHistBytes);
@@ -874,8 +907,7 @@ vx_status radix_prefix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStr
   (first == 4 ? rx_byte_hist<4, 4> : rx_byte_hist<5, 3>)<<<g, kRxThreads, 0, s>>>(b.keys[0], n, bh);
   rx_init<<<8 - first, kRxDigits, 0, s>>>(st, bh, bases, n, spin_limit ? spin_limit : kRxSpinLimit, first);
   for (int pass = first; pass < 8; ++pass)
-    rx_sweep<kSweepThreads, kSweepItems, uint32_t><<<nt, kSweepThreads, kRxSweepSmem, s>>>(b, st, pass, n, bases,
-                                                                                         tickets, status, false);
+    VX_TRY(enqueue_sweep(b, st, pass, n, bases, tickets, status, false, num_sms, s));
   // the list takes the place of the look-back words: 256 * 8 bytes a tile
   const uint32_t cap = nt * (kRxDigits * 8 / 4);
   const int gf = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms * 8);

@@ -1,5 +1,5 @@
-"""The radix sort's scatter at the edges of its 7,168-pair tile, of a warp's
-512 pairs and of a round's 32, on keys whose digits are random, all equal but
+"""The radix sort's scatter at the edges of its 7,168-pair tile (3,584 for a
+small sort), of a warp's pairs and of a round's 32, on keys whose digits are random, all equal but
 one, few, or all ones (the pad of a last tile), against a stable sort by the
 host (exact)."""
 import numpy as np
@@ -10,6 +10,7 @@ pytestmark = pytest.mark.gpu
 vx = pytest.importorskip("paper_2502_09541_gb300")
 
 TILE = 7168
+SMALL = 3584
 
 
 @pytest.fixture(scope="module")
@@ -33,7 +34,8 @@ def _keys(kind, n):
 
 
 @pytest.mark.parametrize("kind", ["random", "few", "one_off", "ones"])
-@pytest.mark.parametrize("n", [1, 31, 33, 511, 513, TILE - 1, TILE, TILE + 1, 2 * TILE, 300 * TILE + 17, 1_000_000])
+@pytest.mark.parametrize("n", [1, 31, 33, 511, 513, TILE - 1, TILE, TILE + 1, 2 * TILE, 300 * TILE + 17, 1_000_000,
+                               SMALL - 1, SMALL, SMALL + 1, 152 * SMALL, 152 * SMALL + 1])
 def test_tile_edges(ctx, kind, n):
     k, v = _keys(kind, n), np.arange(n, dtype=np.uint32)
     ok, ov = vx.vx_radix_sort_pairs(ctx, k, v)
