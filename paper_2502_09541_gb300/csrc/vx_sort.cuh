@@ -16,16 +16,17 @@ RadixState *radix_state_of(char *temp);
 // spin_limit: polls of one predecessor's look-back word before the pass gives
 // up and sets the error word (0 = the default of 2^20).  iota: the values are
 // the positions 0 .. n - 1, which need not be in b.vals[0] (when every pass is
-// skipped they are still nowhere)
+// skipped they are still nowhere).  vals: recorded where the values are copied
+// on another stream; waited for when only they are missing
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass = 8,
-                             uint32_t spin_limit = 0, bool iota = false);
+                             uint32_t spin_limit = 0, bool iota = false, cudaEvent_t vals = nullptr);
 // The same for n < 2^32 pairs whose keys nearly all differ in their upper bytes:
 // passes over the key bytes first .. 7 only, then the few groups of pairs that
 // agree in all of those are put in order where they are.  If a group is large
 // or there are many, bit 17 of the published word says that the pairs (a
 // stable rearrangement of the input) have to be sorted in full.
 vx_status radix_prefix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int first,
-                                    uint32_t spin_limit);
+                                    uint32_t spin_limit, cudaEvent_t vals = nullptr);
 // after radix_sort_enqueue on s: publishes to a mapped host word the buffer
 // holding the result (low byte), the executed passes (next byte), whether
 // a look-back wait gave up (bit 16) and the prefix sort's bit 17
