@@ -89,21 +89,25 @@ __global__ void __launch_bounds__(kMlpThreads, 2) mlp_fwd_bwd_kernel(const float
 // 32 points, lane j of it hidden unit j; the 32 outputs are summed over the
 // units by a transposing butterfly (31 shuffles, and lane k ends with point
 // k's), each lane adds up its unit's three partial derivatives over the points,
-// the block its warps', and writes its 98 sums; behind the barrier every block
-// adds up all blocks' sums in the same order and applies the same update to its
-// own copy of the parameters and moments.  The sums' buffers alternate, so a
-// block can run at most one barrier ahead of the slowest reader.  300 steps on
-// 65,536 points: 5.2 ms as a launch per step in captured graphs (a warp walked
-// its points one by one, 98 global atomics per block, the update in the last
-// block), 1.97 ms now, 6 us a step: a quarter each for the sigmoids, the
-// gradient sums, the barrier and its L2 round trips, and the update.
+// the block its warps', and writes its 97 sums as one row; behind the barrier
+// every block adds up all blocks' rows in the same order and applies the same
+// update to its own copy of the parameters and moments.  The rows' buffers
+// alternate, so a block can run at most one barrier ahead of the slowest reader.
+// 300 steps on 65,536 points: 5.2 ms as a launch per step in captured graphs (a
+// warp walked its points one by one, 98 global atomics per block, the update in
+// the last block); 1.84 ms for the whole call with the sums written parameter by
+// parameter and a fence in every thread; 1.61 ms now.  Of a step's 10,600 cycles
+// the outputs take 2,700 (two special-function instructions a point and unit:
+// 2,050), the gradient sums 950 and the block's 1,300, the barrier with the read
+// of the rows 4,200 and the update 800.  Sums that carry their step's number and are
+// polled for, added up parameter by parameter in one block each, took 2.2 ms.
 struct TrainArgs {
   float *theta;
   const float *x, *t;
   uint64_t m;
   uint32_t steps;
   float lr, b1, b2, eps;
-  float *part;         // 2 x (3H + 1) x blocks
+  float *part;         // 2 x blocks x train_row(H)
   unsigned int *bar;   // [0] arrivals, [1] nonzero: a barrier wait gave up
 };
 
@@ -118,40 +122,47 @@ __device__ __forceinline__ float sigmoid_step(float v) {
   return fmaf(r, fmaf(-d, r, 1.f), r);
 }
 
+// floats of a block's sums: whole 16-byte words, so that the blocks' rows are
+// written and read in few wide accesses
+constexpr int train_row(int H) { return (3 * H + 1 + 3) / 4 * 4; }
 constexpr int kTrainWarps = 14;  // x 147 blocks: a warp per 32 of the 65,536 points
 constexpr uint32_t kTrainPolls = 1u << 22;
 
 template <int H>
 __global__ void __launch_bounds__(32 * kTrainWarps, 1) mlp_train_kernel(const TrainArgs p) {
   static_assert(H >= 1 && H <= 32, "one hidden unit per lane");
-  constexpr int kParams = 3 * H + 1;
+  constexpr int kParams = 3 * H + 1, kRow = train_row(H), kCols = kRow / 4;
+  constexpr int kGroups = 32 * kTrainWarps / kCols < 17 ? 32 * kTrainWarps / kCols : 17;
   __shared__ __align__(16) float s_x[kTrainWarps][32], s_dy[kTrainWarps][32];
   __shared__ float s_part[kTrainWarps][3 * 32 + 1];
-  __shared__ float s_theta[kParams], s_grad[kParams];
-  __shared__ float s_unit[5][32];  // softplus(omega), its derivative, beta, softplus(alpha), its derivative
+  __shared__ __align__(16) float s_sum[kGroups][kRow];
+  __shared__ float s_unit[6][32];  // softplus(omega), its derivative, beta, softplus(alpha), its derivative, gamma
   __shared__ int s_stop;
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const bool on = lane < (uint32_t)H;
-  const uint32_t k = threadIdx.x;
-  float m1 = 0.f, m2 = 0.f;  // moments of parameter k
-  if (k < kParams) s_theta[k] = p.theta[k];
+  const uint32_t k = threadIdx.x, own = k - 32;  // warp 0 waits at the barrier; the next threads own a parameter each
+  float theta = 0.f, m1 = 0.f, m2 = 0.f;
+  auto unit = [&] {  // what the steps use of it
+    if (own < (uint32_t)H || (own >= 2u * H && own < 3u * H)) {
+      const uint32_t row = own < (uint32_t)H ? 0 : 3;
+      s_unit[row][own % H] = softplusf(theta);
+      s_unit[row + 1][own % H] = sigmoidf(theta);
+    } else {
+      s_unit[own < 3u * H ? 2 : 5][own % H] = theta;
+    }
+  };
+  for (uint32_t i = k; i < 6 * 32; i += 32 * kTrainWarps) (&s_unit[0][0])[i] = 0.f;  // lanes without a unit
+  __syncthreads();
+  if (own < (uint32_t)kParams) {
+    theta = p.theta[own];
+    unit();
+  }
   const uint64_t n_warps = (uint64_t)gridDim.x * kTrainWarps, first = ((uint64_t)blockIdx.x * kTrainWarps + w) * 32;
   const float x0 = first + lane < p.m ? p.x[first + lane] : 0.f, t0 = first + lane < p.m ? p.t[first + lane] : 0.f;
   const float inv_m = 1.f / (float)p.m;
   for (uint32_t step = 1; step <= p.steps; ++step) {
     __syncthreads();  // the parameters are there
-    if (k < 32) {
-      const float om = on ? s_theta[lane] : 0.f;
-      s_unit[0][lane] = on ? softplusf(om) : 0.f;
-      s_unit[1][lane] = on ? sigmoidf(om) : 0.f;
-      s_unit[2][lane] = on ? s_theta[H + lane] : 0.f;
-    } else if (k < 64) {
-      const float al = on ? s_theta[2 * H + lane] : 0.f;
-      s_unit[3][lane] = on ? softplusf(al) : 0.f;
-      s_unit[4][lane] = on ? sigmoidf(al) : 0.f;
-    }
-    __syncthreads();
-    const float uw = s_unit[0][lane], ub = s_unit[2][lane], ua = s_unit[3][lane], gamma = s_theta[3 * H];
+    const float uw = s_unit[0][lane], ub = s_unit[2][lane], ua = s_unit[3][lane], gamma = s_unit[5][0];
     float g_om = 0.f, g_be = 0.f, g_al = 0.f, g_ga = 0.f;
     for (uint64_t base = first; base < p.m; base += n_warps * 32) {
       const bool real = base + lane < p.m;
@@ -205,23 +216,24 @@ __global__ void __launch_bounds__(32 * kTrainWarps, 1) mlp_train_kernel(const Tr
     s_part[w][64 + lane] = g_al * s_unit[4][lane];
     if (lane == 0) s_part[w][96] = g_ga;
     __syncthreads();
-    float *part = p.part + (size_t)(step & 1) * kParams * gridDim.x;
-    if (k < kParams) {
-      const int at = k == 3 * H ? 96 : (int)(k / H) * 32 + (int)(k % H);
+    float *part = p.part + (size_t)(step & 1) * kRow * gridDim.x;
+    if (k < kRow) {
+      const int at = k >= 3 * H ? 96 : (int)(k / H) * 32 + (int)(k % H);
       float sum = 0.f;
+      if (k < kParams) {
 #pragma unroll
-      for (int q = 0; q < kTrainWarps; ++q) sum += s_part[q][at];
-      __stcg(&part[(size_t)k * gridDim.x + blockIdx.x], sum);
+        for (int q = 0; q < kTrainWarps; ++q) sum += s_part[q][at];
+      }
+      __stcg(&part[(size_t)blockIdx.x * kRow + k], sum);
     }
-    const float c1 = 1.f - powf(p.b1, (float)step), c2 = 1.f - powf(p.b2, (float)step);
-    __threadfence();
     __syncthreads();
     if (k == 0) {  // barrier: arrivals only grow, step s ends at s x blocks
+      __threadfence();  // the block's sums, which the barrier above has ordered before it
       atomicAdd(&p.bar[0], 1u);
       const uint32_t want = step * gridDim.x;
       int stop = 0;
       for (uint32_t polls = 0; *(volatile unsigned int *)&p.bar[0] < want; ++polls)
-        if (polls > kTrainPolls || *(volatile unsigned int *)&p.bar[1]) {
+        if (polls > kTrainPolls || (polls % 64 == 63 && *(volatile unsigned int *)&p.bar[1])) {
           p.bar[1] = 1;
           stop = 1;
           break;
@@ -229,43 +241,47 @@ __global__ void __launch_bounds__(32 * kTrainWarps, 1) mlp_train_kernel(const Tr
       __threadfence();
       s_stop = stop;
     }
+    float to_m = 0.f, to_v = 0.f;
+    if (own < (uint32_t)kParams) {  // while warp 0 waits
+      to_m = p.lr / (1.f - powf(p.b1, (float)step));
+      to_v = 1.f / (1.f - powf(p.b2, (float)step));
+    }
     __syncthreads();
     if (s_stop) return;
-    {  // warp w adds up parameters w, w + 14, ...: all loads of five rounds of blocks in flight
-      constexpr int kQ = (kParams + kTrainWarps - 1) / kTrainWarps, kR = 5;
-      float sum[kQ];
+    // a thread per four parameters and kGroups-th block: all its loads in flight
+    if (k < kCols * kGroups) {
+      constexpr int kR = 9;
+      const uint32_t g = k / kCols, c = k % kCols;
+      float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (uint32_t b0 = g; b0 < gridDim.x; b0 += kGroups * kR) {
+        float4 v[kR];
 #pragma unroll
-      for (int j = 0; j < kQ; ++j) sum[j] = 0.f;
-      for (uint32_t b0 = 0; b0 < gridDim.x; b0 += 32 * kR) {
-        float v[kQ][kR];
+        for (int j = 0; j < kR; ++j)
+          v[j] = b0 + j * kGroups < gridDim.x
+                     ? __ldcg(reinterpret_cast<const float4 *>(part + (size_t)(b0 + j * kGroups) * kRow) + c)
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < kQ; ++j)
-#pragma unroll
-          for (int r = 0; r < kR; ++r) {
-            const uint32_t q = w + j * kTrainWarps, b = b0 + 32 * r + lane;
-            v[j][r] = q < (uint32_t)kParams && b < gridDim.x ? __ldcg(&part[(size_t)q * gridDim.x + b]) : 0.f;
-          }
-#pragma unroll
-        for (int j = 0; j < kQ; ++j)
-#pragma unroll
-          for (int r = 0; r < kR; ++r) sum[j] += v[j][r];
+        for (int j = 0; j < kR; ++j) {
+          sum.x += v[j].x;
+          sum.y += v[j].y;
+          sum.z += v[j].z;
+          sum.w += v[j].w;
+        }
       }
-#pragma unroll
-      for (int j = 0; j < kQ; ++j) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], off);
-        if (lane == 0 && w + j * kTrainWarps < (uint32_t)kParams) s_grad[w + j * kTrainWarps] = sum[j];
-      }
+      reinterpret_cast<float4 *>(s_sum[g])[c] = sum;
     }
     __syncthreads();
-    if (k < kParams) {
-      const float g = s_grad[k];
+    if (own < (uint32_t)kParams) {
+      float g = 0.f;
+#pragma unroll
+      for (int q = 0; q < kGroups; ++q) g += s_sum[q][own];
       m1 = p.b1 * m1 + (1.f - p.b1) * g;
       m2 = p.b2 * m2 + (1.f - p.b2) * g * g;
-      s_theta[k] -= p.lr * (m1 / c1) / (sqrtf(m2 / c2) + p.eps);
+      theta -= to_m * m1 / (sqrtf(m2 * to_v) + p.eps);
+      unit();
     }
   }
-  if (blockIdx.x == 0 && k < kParams) p.theta[k] = s_theta[k];  // the thread's own
+  if (blockIdx.x == 0 && own < (uint32_t)kParams) p.theta[own] = theta;
 }
 
 // data-driven initial parameters from the (sorted) training points: unit j is
@@ -362,7 +378,7 @@ static vx_status mlp_alloc(vx_ctx *ctx, uint64_t M, MlpWork &w) {
   w.loss = (float *)(p + 2048);
   w.bar = (unsigned int *)(p + 2048 + 64);
   w.part = (float *)(p + 2048 + 256);
-  static_assert(2 * (3 * 32 + 1) * kFewBlocks * 4 <= 4096 - 2048 - 256, "partial sums of kFewBlocks blocks");
+  static_assert(2 * train_row(32) * kFewBlocks * 4 <= 4096 - 2048 - 256, "partial sums of kFewBlocks blocks");
   char *q = p + 4096;
   w.x = (float *)q;
   w.t = (float *)(q + ((4 * M + 255) & ~255ull));
@@ -419,7 +435,7 @@ static vx_status train(vx_ctx *ctx, int H, MlpWork &w, uint64_t m, uint32_t step
   TrainArgs a{w.theta, w.x, w.t, m, steps, lr, 0.9f, 0.999f, 1e-8f, w.part, w.bar};
   if (grid > kFewBlocks) {
     part.arena = &ctx->arena;
-    part.p = ctx->arena.alloc(2ull * (3 * H + 1) * grid * 4);
+    part.p = ctx->arena.alloc(2ull * train_row(H) * grid * 4);
     if (part.p) a.part = part.as<float>();
     else grid = kFewBlocks;
   }
