@@ -266,6 +266,7 @@ __device__ __forceinline__ void rj_for_tuples(RjSegs &s, const uint32_t *bnd, co
     const uint32_t m = nchunks - c0 < (uint32_t)kRjThreads ? nchunks - c0 : (uint32_t)kRjThreads;
     const uint64_t total = s.start[m];
     const uint64_t lo = o0 > done ? o0 - done : 0, hi = o1 - done < total ? o1 - done : total;
+    uint32_t a = 0;  // the chunk of the thread's latest tuple: its ordinals only grow
     for (uint64_t i0 = lo; i0 < hi; i0 += kU * kRjThreads) {
       uint32_t ch[kU];
       uint64_t ix[kU];
@@ -275,10 +276,13 @@ __device__ __forceinline__ void rj_for_tuples(RjSegs &s, const uint32_t *bnd, co
         ix[u] = ~0ull;
         ch[u] = 0;
         if (i < hi) {
-          uint32_t a = 0, b = m - 1;  // the last chunk that starts at or before i
-          while (a < b) {
-            const uint32_t mid = (a + b + 1) / 2;
-            if (s.start[mid] <= i) a = mid; else b = mid - 1;
+          // the last chunk that starts at or before i: mostly the same or the next
+          if (i >= s.start[a + 1] && i >= s.start[++a + 1]) {
+            uint32_t b = m - 1;
+            for (++a; a < b;) {
+              const uint32_t mid = (a + b + 1) / 2;
+              if (s.start[mid] <= i) a = mid; else b = mid - 1;
+            }
           }
           ch[u] = c0 + a;
           ix[u] = s.at[a] + (i - s.start[a]);
@@ -362,8 +366,12 @@ __global__ void __launch_bounds__(kRjThreads) rj_join_kernel(const RjJoinParams 
       rj_for_tuples<4>(segs, p.bbnd, p.bbase, p.nb, ng1, ga, gb, item.y * kRjPart, (item.y + 1ull) * kRjPart,
                        [&](const uint32_t *ch, const uint64_t *ix) {
                          uint64_t k[4];
+                         uint32_t r[4];
 #pragma unroll
-                         for (int u = 0; u < 4; ++u) k[u] = ix[u] == ~0ull ? kRjEmpty : p.bkeys[ix[u]];
+                         for (int u = 0; u < 4; ++u) {
+                           k[u] = ix[u] == ~0ull ? kRjEmpty : p.bkeys[ix[u]];
+                           r[u] = ix[u] == ~0ull ? 0u : p.brows[ix[u]];  // in flight with the keys
+                         }
 #pragma unroll
                          for (int u = 0; u < 4; ++u) {
                            if (ix[u] == ~0ull) continue;
@@ -376,7 +384,7 @@ __global__ void __launch_bounds__(kRjThreads) rj_join_kernel(const RjJoinParams 
                              if (tkey[h] != k[u]) continue;
                              pay = tpay[h];
                            }
-                           const uint64_t row = (uint64_t)ch[u] * p.probe_chunk_rows + p.brows[ix[u]];
+                           const uint64_t row = (uint64_t)ch[u] * p.probe_chunk_rows + r[u];
                            cnt += 1;
                            psum += pay;
                            fp += rj_mix(row ^ ((pay << 17) | (pay >> 47)));
