@@ -145,24 +145,24 @@ struct RjAcc {
   uint32_t err;
 };
 
-// resident mode, after a chunk's clustering: its buffer 1 is the resident
-// array, where the last executed pass of an odd number of them has left the
-// keys (and the probe side's rows); an even number left them in the slot.  The
-// build side's payloads follow in clustered order.
-__global__ void rj_keep_kernel(const RadixBufs b, const RadixState *st, int npass, uint64_t n, const uint64_t *pay,
-                               uint64_t *opay, RjAcc *acc) {
+// resident mode, after a chunk's clustering: buffer `home` is the resident
+// array, where the passes have left the keys (and the probe side's rows) unless
+// an odd number of them was skipped.  The build side's payloads follow in
+// clustered order.
+__global__ void rj_keep_kernel(const RadixBufs b, int home, const RadixState *st, int npass, uint64_t n,
+                               const uint64_t *pay, uint64_t *opay, RjAcc *acc) {
   const int c = st->cur[npass];
   const uint64_t *k = c ? b.keys[1] : b.keys[0];
   const uint32_t *v = c ? b.vals[1] : b.vals[0];
   bool moved = false;
   for (int q = 0; q < npass; ++q) moved = moved || !st->skip[q];
   if (st->err && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&acc->err, ERR_WAIT);
-  if (c && !opay) return;
+  if (c == home && moved && !opay) return;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t row = moved ? v[i] : (uint32_t)i;
-    if (!c) b.keys[1][i] = k[i];
+    if (c != home) b.keys[home][i] = k[i];
     if (opay) opay[i] = pay[row];
-    else b.vals[1][i] = row;
+    else b.vals[home][i] = row;
   }
 }
 
@@ -432,6 +432,7 @@ struct RjPartitionPass : ExKernel {
   const uint64_t *keys, *payload;  // payload null: the probe side (local rows are kept instead)
   uint64_t n, R;
   int bits, npass, S;
+  int first = 0;  // resident: the lowest key byte that the clustering orders by
   uint64_t *mid_keys;
   uint64_t *mid_pay;    // build side
   uint32_t *mid_rows;   // probe side
@@ -461,13 +462,17 @@ struct RjPartitionPass : ExKernel {
     b.vals[1] = (uint32_t *)(slot + 2 * kb() + vb());
     return b;
   }
-  // resident: [keys | rows | rows (build side) | temp | payloads]
+  // resident: [keys | rows | rows (build side) | temp | payloads].  The passes
+  // end in the resident arrays: an odd number starts from the slot, an even one
+  // from the arrays themselves, into which the chunk is then loaded
+  int home() const { return (npass - first) & 1; }
   RadixBufs resident_bufs(char *slot, uint64_t it) const {
+    const int h = home();
     RadixBufs b;
-    b.keys[0] = (uint64_t *)slot;
-    b.keys[1] = mid_keys + it * R;
-    b.vals[0] = (uint32_t *)(slot + kb());
-    b.vals[1] = payload ? (uint32_t *)(slot + kb() + vb()) : mid_rows + it * R;
+    b.keys[1 - h] = (uint64_t *)slot;
+    b.keys[h] = mid_keys + it * R;
+    b.vals[1 - h] = (uint32_t *)(slot + kb());
+    b.vals[h] = payload ? (uint32_t *)(slot + kb() + vb()) : mid_rows + it * R;
     return b;
   }
   char *temp(char *slot) const { return slot + (resident ? 1 : 2) * kb() + 2 * vb(); }
@@ -478,15 +483,16 @@ struct RjPartitionPass : ExKernel {
   }
   uint64_t *pay_out(char *slot) const { return (uint64_t *)((char *)pay_in(slot) + kb()); }
   void inputs(uint64_t it, char *slot, std::vector<CopyOp> &h2d) override {
-    h2d.push_back({keys + it * R, bufs(slot).keys[0], 8 * rows(it)});
+    h2d.push_back({keys + it * R, (resident ? resident_bufs(slot, it) : bufs(slot)).keys[0], 8 * rows(it)});
     if (payload) h2d.push_back({payload + it * R, pay_in(slot), 8 * rows(it)});
   }
   vx_status kernel(char *slot, uint64_t it, cudaStream_t s) override {
     const uint64_t m = rows(it);
     if (resident) {
       const RadixBufs rb = resident_bufs(slot, it);
-      VX_TRY(radix_sort_enqueue(rb, m, temp(slot), s, ctx->num_sms, npass, ctx->cfg.lookback_spin_limit, true));
-      rj_keep_kernel<<<grid_for(ctx, m, 256, 8), 256, 0, s>>>(rb, radix_state_of(temp(slot)), npass, m,
+      VX_TRY(radix_sort_enqueue(rb, m, temp(slot), s, ctx->num_sms, npass, ctx->cfg.lookback_spin_limit, true,
+                                nullptr, first));
+      rj_keep_kernel<<<grid_for(ctx, m, 256, 8), 256, 0, s>>>(rb, home(), radix_state_of(temp(slot)), npass, m,
                                                               payload ? pay_in(slot) : nullptr,
                                                               payload ? mid_pay + it * R : nullptr, acc);
       VX_CUDA_TRY(cudaGetLastError());
@@ -697,6 +703,9 @@ vx_status radix_join_resident(vx_ctx *ctx, const Column *bk, const Column *bp, c
     pp.R = R;
     pp.bits = bits;
     pp.npass = bits / 8;
+    // the join takes whole runs: bytes below a run's first bit need no order
+    // (3M x 30M, runs of 4,096 groups: the call 2.27 -> 2.00 ms)
+    pp.first = std::min(run_shift / 8, pp.npass - 1);
     pp.S = std::max(2, ctx->cfg.n_slots);
     pp.mid_bnd = nullptr;
     pp.mid_keys = (uint64_t *)(m + (side ? rs.bkeys : rs.akeys));
@@ -711,7 +720,7 @@ vx_status radix_join_resident(vx_ctx *ctx, const Column *bk, const Column *bp, c
         pp.mid_keys, n, R, (1ull << bits) - 1, run_shift, n_runs, (uint32_t *)(m + (side ? rs.bbnd : rs.abnd)));
     VX_CUDA_TRY(cudaGetLastError());
     res.bytes_h2d += es.bytes_h2d;
-    res.kernel_launches += es.kernel_launches * (pp.npass + 3) + 1;
+    res.kernel_launches += es.kernel_launches * (pp.npass - pp.first + 3) + 1;
     res.ms_kernel += es.ms_kernel;
   }
   res.ms_partition = res.ms_build = now_ms() - tp;

@@ -921,10 +921,10 @@ static vx_status radix_result(char *temp, cudaStream_t s, int *cur, bool *redo =
 }
 
 // Enqueues a stable LSD radix sort of b.keys[0]/b.vals[0] (n pairs) on s by
-// the low npass bytes of the key (8: the whole key).  The sorted pairs end in
+// the key bytes first .. npass - 1 (0 and 8: the whole key).  The sorted pairs end in
 // buffer st->cur[npass] (0 or 1).
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass,
-                             uint32_t spin_limit, bool iota, cudaEvent_t vals) {
+                             uint32_t spin_limit, bool iota, cudaEvent_t vals, int first) {
   const uint32_t nt = sweep_tiles(n, num_sms);
   RadixState *st = radix_state_of(temp);
   unsigned long long *bh = (unsigned long long *)(temp + kStateBytes);
@@ -939,11 +939,16 @@ vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s
   // histograms, tickets and status words (the words carry their pass number)
   VX_CUDA_TRY(cudaMemsetAsync(bh, 0, kByteHistBytes + kBasesBytes + kTicketBytes + (uint64_t)kRxDigits * nt * 8, s));
   const int g = (int)std::min<uint64_t>((n + kRxThreads - 1) / kRxThreads, (uint64_t)num_sms * 6);
-  auto hist = npass == 1 ? rx_byte_hist<1> : npass == 2 ? rx_byte_hist<2> : npass == 3 ? rx_byte_hist<3> : rx_byte_hist<8>;
+  auto hist = first == 1   ? (npass == 2 ? rx_byte_hist<1, 1> : rx_byte_hist<2, 1>)
+              : first == 2 ? rx_byte_hist<1, 2>
+              : npass == 1 ? rx_byte_hist<1>
+              : npass == 2 ? rx_byte_hist<2>
+              : npass == 3 ? rx_byte_hist<3>
+                           : rx_byte_hist<8>;
   hist<<<g, kRxThreads, 0, s>>>(b.keys[0], n, bh);
-  rx_init<<<npass, kRxDigits, 0, s>>>(st, bh, bases, n, spin_limit ? spin_limit : kRxSpinLimit, 0);
+  rx_init<<<npass - first, kRxDigits, 0, s>>>(st, bh, bases, n, spin_limit ? spin_limit : kRxSpinLimit, first);
   if (vals) VX_CUDA_TRY(cudaStreamWaitEvent(s, vals, 0));
-  for (int pass = 0; pass < npass; ++pass)  // a skipped pass returns at once and keeps the buffer
+  for (int pass = first; pass < npass; ++pass)  // a skipped pass returns at once and keeps the buffer
     VX_TRY(enqueue_sweep(b, st, pass, n, bases, tickets, status, iota, num_sms, s));
   VX_CUDA_TRY(cudaGetLastError());
   return VX_OK;

@@ -17,9 +17,11 @@ RadixState *radix_state_of(char *temp);
 // up and sets the error word (0 = the default of 2^20).  iota: the values are
 // the positions 0 .. n - 1, which need not be in b.vals[0] (when every pass is
 // skipped they are still nowhere).  vals: recorded where the values are copied
-// on another stream; waited for when only they are missing
+// on another stream; waited for when only they are missing.  first: the lowest
+// key byte that counts (0; 1 or 2 with at most three passes)
 vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int npass = 8,
-                             uint32_t spin_limit = 0, bool iota = false, cudaEvent_t vals = nullptr);
+                             uint32_t spin_limit = 0, bool iota = false, cudaEvent_t vals = nullptr,
+                             int first = 0);
 // The same for n < 2^32 pairs whose keys nearly all differ in their upper bytes:
 // passes over the key bytes first .. 7 only, then the few groups of pairs that
 // agree in all of those are put in order where they are.  If a group is large

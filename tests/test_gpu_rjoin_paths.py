@@ -70,3 +70,19 @@ def test_pieces_hot_key_and_ones(budget):
         with pytest.raises(vx.VxError) as e:
             _run(k2, k2, pk, budget)
         assert e.value.status == vx.VX_E_DUPKEY
+
+
+@pytest.mark.parametrize("bits", [8, 16, 24])
+@pytest.mark.parametrize("nb", [700, 768 * 200, 768 * 400])
+def test_resident_clustering_by_upper_bytes(nb, bits):
+    """Builds whose runs of groups need one to three clustered bytes; keys
+    that share a byte (a pass left out) and keys that share all of them."""
+    npr = 1_500_007
+    base = np.random.default_rng(nb).permutation(nb).astype(np.int64)
+    for shift in (0, 8, 16):
+        bk = base << shift | 3 << 50
+        bp = (base * 7 + 1).astype(np.int64)
+        pk = np.random.default_rng(2).choice(bk, npr)
+        pk[::5] += 1 << 55
+        r = _check(bk, bp, pk, 4096, bits)
+        assert r["bytes_d2h"] == 0
