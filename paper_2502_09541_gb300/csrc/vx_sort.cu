@@ -1485,9 +1485,12 @@ uint64_t resident_left(uint64_t n, uint64_t m, uint32_t P, uint64_t avail) {
 // Partitions requested so that two slots of pass 2 fit what the regions leave,
 // with room for uneven partitions; 0: they do not fit.
 uint32_t resident_partitions(uint64_t n, uint64_t m, uint64_t avail, double headroom) {
-  // at most 12M pairs a job, so that the stores start early
-  double P = std::max(4.0, std::ceil((double)n / 12e6));
-  for (int i = 0; i < 8 && P <= 64; ++i) {
+  // at most 12M pairs a job as far as kMaxResident partitions go, so that the
+  // stores start early (1e9 pairs under 16 GiB: 122 ms with 64 resident
+  // partitions, 162 through host memory)
+  constexpr double kMaxResident = 64.0;
+  double P = std::min(kMaxResident, std::max(4.0, std::ceil((double)n / 12e6)));
+  for (int i = 0; i < 8 && P <= kMaxResident; ++i) {
     const double jcap = (double)resident_left(n, m, (uint32_t)P, avail) / (2 * 12.6);
     if (jcap < 1) return 0;
     if (headroom * (double)n / jcap <= P) return (uint32_t)P;
