@@ -304,8 +304,15 @@ std::mutex g_addr_mu;
 uint32_t *g_addr[64] = {};
 uint64_t g_calls[64] = {};
 int g_pageable[64] = {};  // the device accesses pageable host memory through the host's page tables
+// Where a device with g_pageable stores the last call's count and error.  They
+// outlive the call: a kernel whose call returned early (a wait for the stream
+// that failed, say because the stream is being captured) may still store them.
+struct alignas(64) HostResult {
+  volatile uint64_t w[2];
+};
+HostResult g_result[64];
 
-vx_status scratch_address(uint32_t **out, uint64_t *call, bool *pageable) {
+vx_status scratch_address(uint32_t **out, uint64_t *call, volatile uint64_t **host_res) {
   int dev = 0;
   VX_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) {
@@ -325,7 +332,7 @@ vx_status scratch_address(uint32_t **out, uint64_t *call, bool *pageable) {
     g_addr[dev] = (uint32_t *)p;
   }
   *out = g_addr[dev];
-  *pageable = g_pageable[dev] != 0;
+  *host_res = g_pageable[dev] ? g_result[dev].w : nullptr;
   *call = g_calls[dev] = (g_calls[dev] + 1) % kSfCalls;
   return VX_OK;
 }
@@ -389,30 +396,31 @@ VX_API vx_status vx_filter_device_static(const int32_t *const *cols, int32_t n_c
   *out_count = 0;
   if (n_rows == 0) return VX_OK;
   uint32_t *scratch = nullptr;
-  bool pageable = false;
-  VX_TRY(scratch_address(&scratch, &p.call, &pageable));
+  volatile uint64_t *host_res = nullptr;
+  VX_TRY(scratch_address(&scratch, &p.call, &host_res));
   cudaStream_t s = (cudaStream_t)stream;
   if (p.call == 0) VX_CUDA_TRY(cudaMemsetAsync(scratch, 0, 4ull * kStaticScratchWords, s));  // the numbers start again
   const bool large = n_rows > kSfLargeRows;
   const uint64_t tile = (large ? kSfLarge : kSfSmall) * kSfGroupRows;
   p.n_tiles = (uint32_t)((n_rows + tile - 1) / tile);
   const bool scan = p.n_tiles > kSfLookBackTiles;
-  // the kernel writes the count to this thread's stack where the GPU reads and
+  // the kernel writes the count to host memory itself where the GPU reads and
   // writes pageable host memory through the host's page tables (a copy of 16
   // bytes back from the device took 8 us more of a 21 us call)
-  volatile uint64_t host_res[2] = {0, 0};
-  p.result = pageable ? (uint64_t *)host_res : (uint64_t *)(scratch + kSfControl + 4);
+  if (host_res) host_res[0] = host_res[1] = 0;
+  p.result = host_res ? (uint64_t *)host_res : (uint64_t *)(scratch + kSfControl + 4);
   auto kernel = large  ? (vec ? sf_filter_kernel<true, kSfLarge, true> : sf_filter_kernel<false, kSfLarge, true>)
                 : scan ? (vec ? sf_filter_kernel<true, kSfSmall, true> : sf_filter_kernel<false, kSfSmall, true>)
                        : (vec ? sf_filter_kernel<true, kSfSmall, false> : sf_filter_kernel<false, kSfSmall, false>);
+  cudaGetLastError();  // an error that an earlier call of this thread left is not this launch's
   kernel<<<p.n_tiles + (scan ? 1 : 0), kSfThreads, 0, s>>>(p, scratch, out_rows);
   VX_CUDA_TRY(cudaGetLastError());
   uint64_t res[2] = {0, 0};
-  if (!pageable) VX_CUDA_TRY(cudaMemcpyAsync(res, p.result, sizeof res, cudaMemcpyDeviceToHost, s));
+  if (!host_res) VX_CUDA_TRY(cudaMemcpyAsync(res, p.result, sizeof res, cudaMemcpyDeviceToHost, s));
   VX_CUDA_TRY(cudaStreamSynchronize(s));
-  const uint64_t total = pageable ? host_res[0] : res[0];
-  if (pageable ? host_res[1] : res[1]) {
-    if (!pageable) VX_CUDA_TRY(cudaMemsetAsync(p.result, 0, sizeof res, s));
+  const uint64_t total = host_res ? host_res[0] : res[0];
+  if (host_res ? host_res[1] : res[1]) {
+    if (!host_res) VX_CUDA_TRY(cudaMemsetAsync(p.result, 0, sizeof res, s));
     set_error("vx_filter_device_static: a look-back wait gave up");
     return VX_E_TIMEOUT;
   }
