@@ -44,6 +44,12 @@ constexpr uint32_t kStaticScratchWords = 65536 + 64;
 // the tickets (call number and count) and the result: count, error (64 bits each)
 constexpr uint32_t kSfControl = 65536;
 constexpr uint32_t kSfSpinLimit = 1u << 20;  // polls of a window of predecessor words before giving up
+// Polls after which a tile stops counting on the scan block and looks back
+// itself (about 0.1 ms; a tile of a call that has the GPU waits some 10 us), and
+// after which the scan block gives its place up (about 50 ms: it waits for
+// tiles that may not have started, which only costs time where it holds the
+// last free place).
+constexpr uint32_t kSfOwnPolls = 128, kSfScanPolls = 1u << 16;
 static_assert(2 * kStaticMaxTiles <= kSfControl, "a look-back word per tile");
 static_assert(kSfLarge * kSfGroupRows <= 65536, "tile rows fit 16 bits");
 
@@ -104,46 +110,41 @@ __device__ __forceinline__ uint32_t sf_look_back(const volatile uint64_t *words,
 }
 
 // The scan block of a call with many tiles: its warps take windows of 32
-// tiles in turn, wait for the tiles' counts, add them up behind the window
+// tiles in turn, wait for the tiles' words, add their counts up behind the window
 // before (a carry handed from warp to warp in shared memory) and replace every
-// count by the tile's exclusive prefix, so that the prefixes advance by a
-// window per hand-over instead of a window per round trip to memory.
+// word by the count of everything up to the tile, so that the prefixes advance by
+// a window per hand-over instead of a window per round trip to memory.  A tile
+// that has looked back itself has left that count already.
 __device__ __forceinline__ void sf_scan_block(const SfParams &p, volatile uint64_t *words) {
   // carry into window k at [k % 16], tagged with k + 1 (at most 8 windows are in work)
   __shared__ uint64_t s_carry[2 * kSfWarps];
   if (threadIdx.x < 2 * kSfWarps) s_carry[threadIdx.x] = threadIdx.x == 0 ? 1ull << 32 : 0ull;
   __syncthreads();
   volatile uint64_t *carry = s_carry;
+  constexpr uint32_t kWhole = 1u << 31;  // the sum counts from the first tile on, not from the window's
   const uint32_t lane = threadIdx.x & 31, n_win = (p.n_tiles + 31) / 32;
   for (uint32_t k = threadIdx.x >> 5; k < n_win; k += kSfWarps) {
     const uint32_t t = 32 * k + lane;
-    uint32_t v = 0;
+    uint32_t x = 0;
     for (uint32_t polls = 0;; ++polls) {
       const uint64_t w = t < p.n_tiles ? words[t] : sf_word(p.call, kSfAgg, 0);
-      v = sf_value(w);
-      if (__all_sync(0xffffffffu, sf_flag(w, p.call) != 0)) break;
-      if (polls > kSfSpinLimit) {
-        if (lane == 0) p.result[1] = 1;
-        return;
-      }
+      const uint32_t flag = sf_flag(w, p.call);
+      x = sf_value(w) | (flag == kSfIncl ? kWhole : 0u);
+      if (__all_sync(0xffffffffu, flag != 0)) break;
+      if (polls > kSfScanPolls) return;  // the tiles manage without
     }
-    uint32_t x = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= (uint32_t)o) x += y;
+      if (lane >= (uint32_t)o && !(x & kWhole)) x += y;
     }
     uint64_t c = carry[k % (2 * kSfWarps)];
     for (uint32_t polls = 0; (uint32_t)(c >> 32) != k + 1; c = carry[k % (2 * kSfWarps)])
-      if (++polls > 64 * kSfSpinLimit) {
-        if (lane == 0) p.result[1] = 1;
-        return;
-      }
-    const uint32_t in = (uint32_t)c, out = in + __shfl_sync(0xffffffffu, x, 31);
+      if (++polls > 64 * kSfScanPolls) return;
+    x = x & kWhole ? x & ~kWhole : (uint32_t)c + x;
     __syncwarp();
-    if (lane == 0) carry[(k + 1) % (2 * kSfWarps)] = (uint64_t)(k + 2) << 32 | out;
-    if (t < p.n_tiles) words[t] = sf_word(p.call, kSfIncl, in + x - v);
-    if (k + 1 == n_win && lane == 0) p.result[0] = out;
+    if (lane == 31) carry[(k + 1) % (2 * kSfWarps)] = (uint64_t)(k + 2) << 32 | x;
+    if (t < p.n_tiles) words[t] = sf_word(p.call, kSfIncl, x);
   }
 }
 
@@ -157,7 +158,9 @@ __device__ __forceinline__ void sf_scan_block(const SfParams &p, volatile uint64
 // in order; the tile's first output position comes from a look-back over its
 // predecessors' words, or with kScan from the block with the first ticket, which
 // does nothing but turn the tiles' counts into prefixes; then the survivors leave
-// as one contiguous run.  Three columns of 2^26 rows, 2 % qualifying: 171 us
+// as one contiguous run.  The scan block works on whole windows, whose later
+// tiles may not have a place on the GPU yet, so a tile whose prefix does not come
+// looks back itself: no tile needs one that has not started.  Three columns of 2^26 rows, 2 % qualifying: 171 us
 // for the call, of which 20 us are not the kernel (5.4 TB/s, 0.79 of the
 // measured copy bandwidth); 907 us when a count pass, a scan of the tiles and a
 // write pass read the columns twice in 4-byte loads.  10,007 rows, two columns:
@@ -255,7 +258,7 @@ __global__ void __launch_bounds__(kSfThreads) sf_filter_kernel(const SfParams p,
     }
     if (lane == 0) {
       s_total = total;
-      words[tile] = sf_word(p.call, kScan || tile ? kSfAgg : kSfIncl, total);
+      words[tile] = sf_word(p.call, tile ? kSfAgg : kSfIncl, total);
     }
     if (!kScan) {
       bool gave_up = false;
@@ -279,17 +282,31 @@ __global__ void __launch_bounds__(kSfThreads) sf_filter_kernel(const SfParams p,
       for (int j = 0; j < 4; ++j)
         if (keep[b] >> (4 * g + j) & 1u) s_row[at++] = (uint16_t)(r + j);
     }
-  if (kScan && threadIdx.x == 0) {
-    uint64_t w = words[tile];
-    for (uint32_t polls = 0; sf_flag(w, p.call) != kSfIncl; w = words[tile]) {
-      if (++polls > kSfSpinLimit) {
-        p.result[1] = 1;
-        s_total = 0;  // nothing is written
-        break;
-      }
+  if (kScan && warp == 0) {
+    const uint32_t total = s_total;
+    uint64_t w = 0;
+    for (uint32_t polls = 0; polls < kSfOwnPolls; ++polls) {
+      w = __shfl_sync(0xffffffffu, words[tile], 0);
+      if (sf_flag(w, p.call) == kSfIncl) break;
       __nanosleep(200);
     }
-    s_prefix = sf_value(w);
+    uint32_t prefix = sf_value(w) - total;
+    if (sf_flag(w, p.call) != kSfIncl) {
+      bool gave_up = false;
+      prefix = sf_look_back(words, p.call, tile, lane, &gave_up);
+      if (lane == 0) {
+        if (gave_up) {
+          p.result[1] = 1;
+          s_total = 0;  // nothing is written
+        } else {
+          words[tile] = sf_word(p.call, kSfIncl, prefix + total);
+        }
+      }
+    }
+    if (lane == 0) {
+      if (tile == p.n_tiles - 1) p.result[0] = prefix + total;
+      s_prefix = prefix;
+    }
   }
   __syncthreads();
   const uint64_t pos0 = s_prefix;
