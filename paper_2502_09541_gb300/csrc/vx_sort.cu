@@ -22,6 +22,7 @@
 #include <thread>
 
 #include "vx_internal.h"
+#include "vx_prefix.cuh"
 #include "vx_radix.cuh"
 #include "vx_sort.cuh"
 
@@ -580,61 +581,32 @@ __global__ void rx_publish(const RadixState *st, int pass, uint64_t *host_word) 
                (uint64_t)(st->redo != 0) << 17;
 }
 
-// ---- prefix sort: the pairs are in the order of their keys' bytes first .. 7;
-// what is left are groups of equal prefix whose low bytes descend somewhere
-constexpr uint32_t kFixGroup = 16;  // pairs of a group that one thread repairs
+// ---- prefix sort: what the passes over the upper key bytes left out of order
+// (vx_prefix.cuh)
 
-// lists the first pair of every group with a descent (found by the group's
-// first one); a group of more than kFixGroup pairs, or a full list, asks for the
-// sort in full
-__global__ void rx_find_kernel(const RadixBufs b, RadixState *st, uint32_t n, int shift, uint32_t *list, uint32_t cap) {
+// lists the first pair of every group to repair; a group of more than kFixGroup
+// pairs, or a full list, asks for the sort in full
+__global__ void rx_find_kernel(const RadixBufs b, RadixState *st, uint64_t n, int shift, uint32_t *list, uint32_t cap) {
   const uint64_t *k = st->cur[8] ? b.keys[1] : b.keys[0];
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i + 1 < n; i += gridDim.x * blockDim.x) {
-    const uint64_t a = k[i], c = k[i + 1];
-    if (a <= c || a >> shift != c >> shift) continue;
-    uint32_t j = i, e = i + 2;
-    bool mine = true;
-    for (uint64_t x = a; mine && j > 0; --j) {  // back to the group's first pair, or to an earlier descent
-      const uint64_t y = k[j - 1];
-      if (y >> shift != a >> shift) break;
-      mine = y <= x && i - j < kFixGroup;
-      if (y <= x && !mine) st->redo = 1;
-      x = y;
-    }
-    while (mine && e < n && k[e] >> shift == a >> shift) {
-      if (++e - j > kFixGroup) {
-        st->redo = 1;
-        mine = false;
-      }
-    }
-    if (!mine) continue;
-    const uint32_t at = atomicAdd(&st->n_fix, 1u);
-    if (at < cap) list[at] = j;
+  for (PrefixWalk w{blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, n, (uint64_t)gridDim.x * blockDim.x}; w.more();
+       w.next()) {
+    uint64_t first = 0;
+    const PrefixFind what = prefix_find(k, n, w.i, shift, &first);
+    if (what == kFixNone) continue;
+    const uint32_t at = what == kFixList ? atomicAdd(&st->n_fix, 1u) : cap;
+    if (at < cap) list[at] = (uint32_t)first;
     else st->redo = 1;
   }
 }
 
-// a thread per listed group: a stable insertion sort where the group is
-__global__ void rx_fix_kernel(const RadixBufs b, const RadixState *st, uint32_t n, int shift, const uint32_t *list,
+// a thread per listed group
+__global__ void rx_fix_kernel(const RadixBufs b, const RadixState *st, uint64_t n, int shift, const uint32_t *list,
                               uint32_t cap) {
   uint64_t *k = st->cur[8] ? b.keys[1] : b.keys[0];
   uint32_t *v = st->cur[8] ? b.vals[1] : b.vals[0];
   const uint32_t m = st->n_fix < cap ? st->n_fix : cap;
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < m; q += gridDim.x * blockDim.x) {
-    const uint32_t j = list[q];
-    const uint64_t prefix = k[j] >> shift;
-    for (uint32_t e = j + 1; e < n && k[e] >> shift == prefix; ++e) {
-      const uint64_t x = k[e];
-      const uint32_t y = v[e];
-      uint32_t at = e;
-      for (; at > j && k[at - 1] > x; --at) {
-        k[at] = k[at - 1];
-        v[at] = v[at - 1];
-      }
-      k[at] = x;
-      v[at] = y;
-    }
-  }
+  for (uint64_t q = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; q < m; q += (uint64_t)gridDim.x * blockDim.x)
+    prefix_fix(k, v, n, list[q], shift);
 }
 
 // ---- sampling and splitters -----------------------------------------------
@@ -975,8 +947,8 @@ vx_status radix_prefix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStr
   // the list takes the place of the look-back words: 256 * 8 bytes a tile
   const uint32_t cap = nt * (kRxDigits * 8 / 4);
   const int gf = (int)std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms * 8);
-  rx_find_kernel<<<gf, 256, 0, s>>>(b, st, (uint32_t)n, 8 * first, (uint32_t *)status, cap);
-  rx_fix_kernel<<<num_sms * 2, 256, 0, s>>>(b, st, (uint32_t)n, 8 * first, (const uint32_t *)status, cap);
+  rx_find_kernel<<<gf, 256, 0, s>>>(b, st, n, 8 * first, (uint32_t *)status, cap);
+  rx_fix_kernel<<<num_sms * 2, 256, 0, s>>>(b, st, n, 8 * first, (const uint32_t *)status, cap);
   VX_CUDA_TRY(cudaGetLastError());
   return VX_OK;
 }
