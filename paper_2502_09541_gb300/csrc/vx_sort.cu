@@ -2065,16 +2065,26 @@ VX_API vx_status vx_radix_sort_pairs(vx_ctx *ctx, const uint64_t *keys, const ui
   b.vals[1] = (uint32_t *)(p + 2 * kb + vb);
   char *temp = p + 2 * kb + 2 * vb;
   cudaStream_t s = ctx->s_compute;
-  VX_CUDA_TRY(cudaMemcpyAsync(b.keys[0], keys, 8 * n, cudaMemcpyHostToDevice, s));
-  struct Event {
+  const bool sample = n >= kPairSampleMin && n >> 32 == 0;
+  // Where the keys are sampled, the values cross the link on the other stream
+  // meanwhile: behind all that the compute stream was given before this call
+  // (which may still use the arena), and waited for before the block goes back
+  // to the arena, also when the call ends early.
+  struct ValsIn {
+    cudaStream_t other;
     cudaEvent_t e = nullptr;
-    ~Event() {
+    bool copying = false;
+    ~ValsIn() {
+      if (copying) cudaStreamSynchronize(other);
       if (e) cudaEventDestroy(e);
     }
-  } vals_in;
-  VX_CUDA_TRY(cudaEventCreateWithFlags(&vals_in.e, cudaEventDisableTiming));
-  // The values cross the link while the keys are sampled and their digits counted.
-  const bool sample = n >= kPairSampleMin && n >> 32 == 0;
+  } vals_in{ctx->s_h2d};
+  if (sample) {
+    VX_CUDA_TRY(cudaEventCreateWithFlags(&vals_in.e, cudaEventDisableTiming));
+    VX_CUDA_TRY(cudaEventRecord(vals_in.e, s));
+    VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_h2d, vals_in.e, 0));
+  }
+  VX_CUDA_TRY(cudaMemcpyAsync(b.keys[0], keys, 8 * n, cudaMemcpyHostToDevice, s));
   volatile uint64_t *word = ctx->h_scalars + 64;
   const uint32_t m = (uint32_t)std::min<uint64_t>(n, kPairSample);
   if (sample) {
@@ -2088,10 +2098,11 @@ VX_API vx_status vx_radix_sort_pairs(vx_ctx *ctx, const uint64_t *keys, const ui
     pair_prefix_kernel<<<1, 1024, sizeof(PairSampleSmem), s>>>(b.keys[0], n, m, ctx->d_scalars + 64);
     VX_CUDA_TRY(cudaGetLastError());
   }
-  VX_CUDA_TRY(cudaMemcpyAsync(b.vals[0], vals, 4 * n, cudaMemcpyHostToDevice, ctx->s_h2d));
-  VX_CUDA_TRY(cudaEventRecord(vals_in.e, ctx->s_h2d));
+  VX_CUDA_TRY(cudaMemcpyAsync(b.vals[0], vals, 4 * n, cudaMemcpyHostToDevice, sample ? ctx->s_h2d : s));
   int first = 0;
   if (sample) {
+    vals_in.copying = true;
+    VX_CUDA_TRY(cudaEventRecord(vals_in.e, ctx->s_h2d));
     VX_CUDA_TRY(cudaStreamSynchronize(s));
     const uint64_t c[4] = {word[0], word[1], word[2], word[3]};
     first = prefix_bytes(c, m, n);
@@ -2102,6 +2113,7 @@ VX_API vx_status vx_radix_sort_pairs(vx_ctx *ctx, const uint64_t *keys, const ui
   VX_TRY(first ? radix_prefix_sort_enqueue(b, n, temp, s, ctx->num_sms, first, limit, vals_in.e)
                : radix_sort_enqueue(b, n, temp, s, ctx->num_sms, 8, limit, false, vals_in.e));
   VX_TRY(radix_result(temp, s, &cur, first ? &redo : nullptr));
+  vals_in.copying = false;  // s, which has waited for them, has been waited for
   if (redo) {  // a prefix that many keys share: sort in full, from where the pairs are
     if (cur) {
       std::swap(b.keys[0], b.keys[1]);
