@@ -1543,25 +1543,6 @@ bool resident_layout(uint64_t n, uint64_t m, const std::vector<uint64_t> &spl, c
   return rp->S2 >= 2 && 12 * rp->pairs + sizeof(RxRegions) + 4096 <= rest;
 }
 
-// How many low key bytes (4, 3 or 0) the sorts may leave to a repair, from the
-// sorted sample: keys that differ but agree in all other bytes have to be rare
-// (at most kFixRate of them per key among the n keys), and keys must not repeat
-// much: a repeated key that shares its prefix makes a group too large to repair.
-// Equal sample neighbours beyond the rows drawn twice show keys that repeat
-// throughout, eight equal ones a single frequent key.  The sort checks what it
-// finds, so a sample that misleads costs a second sort of the partition and
-// nothing else.  Partitions of 8.4M uniform keys: four passes and the repair
-// 0.37 ms, eight passes 0.62; the call of 67M pairs 10.2 -> 9.3 ms
-constexpr double kFixRate = 0.06;
-
-int prefix_bytes(const uint64_t (&c)[4], uint64_t m, uint64_t n) {
-  // sample rows that repeat one drawn before: m less the distinct rows drawn
-  const double twice = (double)m + (double)n * std::expm1(-(double)m / (double)n);
-  if (c[2] || (double)c[3] > 1.5 * twice + 6.0 * std::sqrt(twice) + 16.0) return 0;
-  const double per = 2.0 / (double)m * ((double)n / (double)m);  // a pair of sample neighbours, in neighbours per key
-  return (double)c[0] * per <= kFixRate ? 4 : (double)c[1] * per <= kFixRate ? 3 : 0;
-}
-
 // Both passes with resident partitions.  *done = false: a region was too small
 // (nothing has been written to the output; the caller sorts the other way).
 vx_status resident_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals, uint64_t n, uint64_t *out_keys,
@@ -1776,7 +1757,7 @@ static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *v
     }
     VX_TRY(cut(P_in));
     reside = resident_layout(n, m, spl, srank, rest, &rp);
-    if (pbuf.p) first = prefix_bytes(prefix, m, n);
+    if (pbuf.p) first = prefix_bytes(prefix, m, n, false);
     pbuf.release();
     if (!reside) rp.release();
   }
@@ -2105,7 +2086,7 @@ VX_API vx_status vx_radix_sort_pairs(vx_ctx *ctx, const uint64_t *keys, const ui
     VX_CUDA_TRY(cudaEventRecord(vals_in.e, ctx->s_h2d));
     VX_CUDA_TRY(cudaStreamSynchronize(s));
     const uint64_t c[4] = {word[0], word[1], word[2], word[3]};
-    first = prefix_bytes(c, m, n);
+    first = prefix_bytes(c, m, n, true);
   }
   const uint32_t limit = ctx->cfg.lookback_spin_limit;
   int cur = 0;
