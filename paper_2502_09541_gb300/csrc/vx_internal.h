@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/vx.h"
+#include "vx_once.h"
 
 #define VX_API extern "C" __attribute__((visibility("default")))
 
@@ -43,6 +44,21 @@ struct Status {
     vx_status s_ = (expr);        \
     if (s_ != VX_OK) return s_;   \
   } while (0)
+
+// Raises a kernel's limit of dynamic shared memory (48 KB by default) on the
+// current device, once: every device has its own.
+template <class K>
+vx_status raise_smem_limit(OncePerDevice &once, K *kernel, size_t bytes) {
+  int device = 0;
+  VX_CUDA_TRY(cudaGetDevice(&device));
+  cudaError_t limit = cudaSuccess;
+  once.run(device, [&] {
+    limit = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return limit == cudaSuccess;
+  });
+  VX_CUDA_TRY(limit);
+  return VX_OK;
+}
 
 // device error word bits (kernels set them, the host turns them into statuses)
 enum : uint32_t {

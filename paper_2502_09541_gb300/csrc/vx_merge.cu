@@ -1064,12 +1064,8 @@ vx_status tile_merge(vx_ctx *ctx, const uint64_t *rk, const uint32_t *rv, uint64
   mp.out_vals = out_vals;
   mp.S = (int)std::min<uint64_t>(kMaxSortSlots, ctx->arena.largest_free() / ((mp.slot_bytes() + 255) & ~255ull));
   if (mp.S < 2) return VX_OK;
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(tile_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
-  });
-  VX_CUDA_TRY(attr);
+  static OncePerDevice once;
+  VX_TRY(raise_smem_limit(once, tile_merge_kernel, sizeof(TileSmem)));
   ExecStats es;
   VX_TRY(run_pipeline(ctx, mp, &es));
   ss.bytes_d2h += es.bytes_d2h;

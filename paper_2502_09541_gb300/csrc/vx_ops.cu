@@ -288,12 +288,8 @@ vx_status run_star_operators(vx_ctx *ctx, const vx_plan *plan, vx_result *out) {
     op.out_g = g_buf[1 - cur];
     op.out_cnt = counts[1 - cur].data();
     if (op.kind == kOpAggregate && P.n_groups <= kSmemGroups) {
-      static bool attr = false;
-      if (!attr) {
-        VX_CUDA_TRY(cudaFuncSetAttribute(op_stage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(16 * kSmemGroups)));
-        attr = true;
-      }
+      static OncePerDevice once;
+      VX_TRY(raise_smem_limit(once, op_stage_kernel, 16 * kSmemGroups));
     }
     ExecStats es;
     VX_TRY(run_pipeline(ctx, op, &es));

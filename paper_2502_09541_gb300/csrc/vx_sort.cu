@@ -539,13 +539,8 @@ static vx_status launch_sweep(RadixBufs b, RadixState *st, int pass, uint64_t n,
                               unsigned int *tickets, unsigned long long *status, bool iota, uint32_t tiles,
                               cudaStream_t s) {
   constexpr size_t smem = sizeof(RxSweepSmem<kSweepThreads, kI, Off>);
-  static std::once_flag once;
-  static cudaError_t attr = cudaSuccess;
-  std::call_once(once, [] {
-    attr = cudaFuncSetAttribute(rx_sweep<kSweepThreads, kI, Off>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-  });
-  VX_CUDA_TRY(attr);
+  static OncePerDevice once;
+  VX_TRY(raise_smem_limit(once, rx_sweep<kSweepThreads, kI, Off>, smem));
   rx_sweep<kSweepThreads, kI, Off><<<tiles, kSweepThreads, smem, s>>>(b, st, pass, n, bases, tickets, status, iota);
   return VX_OK;
 }
@@ -560,15 +555,9 @@ static vx_status enqueue_sweep(RadixBufs b, RadixState *st, int pass, uint64_t n
   return launch_sweep<16, uint32_t>(b, st, pass, n, bases, tickets, status, iota, nt, s);
 }
 
-// the scatters' shared memory is above the 48 KB default: raise the limit once
 static vx_status rx_scatter_attr() {
-  static bool done = false;
-  if (!done) {
-    VX_CUDA_TRY(cudaFuncSetAttribute(rx_range_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kRxScatterSmem));
-    done = true;
-  }
-  return VX_OK;
+  static OncePerDevice once;
+  return raise_smem_limit(once, rx_range_scatter, kRxScatterSmem);
 }
 
 // publishes the buffer holding the result (low byte), the number of
@@ -2069,13 +2058,8 @@ VX_API vx_status vx_radix_sort_pairs(vx_ctx *ctx, const uint64_t *keys, const ui
   volatile uint64_t *word = ctx->h_scalars + 64;
   const uint32_t m = (uint32_t)std::min<uint64_t>(n, kPairSample);
   if (sample) {
-    static std::once_flag once;
-    static cudaError_t attr = cudaSuccess;
-    std::call_once(once, [] {
-      attr = cudaFuncSetAttribute(pair_prefix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(PairSampleSmem));
-    });
-    VX_CUDA_TRY(attr);
+    static OncePerDevice once;
+    VX_TRY(raise_smem_limit(once, pair_prefix_kernel, sizeof(PairSampleSmem)));
     pair_prefix_kernel<<<1, 1024, sizeof(PairSampleSmem), s>>>(b.keys[0], n, m, ctx->d_scalars + 64);
     VX_CUDA_TRY(cudaGetLastError());
   }

@@ -709,13 +709,9 @@ static int vec_resident(size_t smem) {
 template <bool kSmem, bool kSplit, int kR>
 static vx_status launch_vec_w(const vx_ctx *ctx, const ChunkParams &p, uint64_t n, size_t acc_smem,
                               cudaStream_t s) {
-  static bool attr = false;  // the largest dynamic size this instantiation takes
-  if (!attr) {
-    VX_CUDA_TRY(cudaFuncSetAttribute(star_vec_kernel<kSmem, kSplit, kR>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)((kSmem ? 16 * kSmemGroups : 0) + vec_col_bytes(kSplit, kR))));
-    attr = true;
-  }
+  static OncePerDevice once;  // the largest dynamic size this instantiation takes
+  VX_TRY(raise_smem_limit(once, star_vec_kernel<kSmem, kSplit, kR>,
+                          (kSmem ? 16 * kSmemGroups : 0) + vec_col_bytes(kSplit, kR)));
   const size_t smem = acc_smem + vec_col_bytes(kSplit, kR);
   constexpr uint64_t kTile = (uint64_t)vec_groups(kSplit, kR) * kVecTileRows;
   uint64_t grid = (n + kTile - 1) / kTile;
@@ -753,17 +749,13 @@ static vx_status launch_bulk(const vx_ctx *ctx, const ChunkParams &p, size_t acc
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     cudaGetLastError();
   });
-  static bool attr = false;
+  static OncePerDevice raised;
   constexpr size_t kStatic = 1024;  // the kernel's static shared memory, rounded up
   if (smem_optin <= (int)kStatic || smem_sm <= 0) {
     set_error("launch_bulk: shared-memory limits unavailable");
     return VX_E_CUDA;
   }
-  if (!attr) {
-    VX_CUDA_TRY(cudaFuncSetAttribute(star_bulk_kernel<kSmem, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     smem_optin - (int)kStatic));
-    attr = true;
-  }
+  VX_TRY(raise_smem_limit(raised, star_bulk_kernel<kSmem, kSplit>, smem_optin - kStatic));
   const uint32_t nr = (uint32_t)p.n_rowroles;
   const size_t stage = (size_t)nr * kBulkColBytes;
   const int bps = std::max(1, std::min(8, ctx->cfg.blocks_per_sm));
@@ -1004,11 +996,11 @@ vx_status launch_star_scan(vx_ctx *ctx, const ChunkParams *d_params, uint32_t n_
                            uint64_t col_stride, uint32_t n_cols, uint64_t n_rows, unsigned int *d_next,
                            cudaStream_t s) {
   if (!n_q || !n_rows || !n_cols) return VX_OK;
+  static OncePerDevice once;
   static int occ = 0;
   const size_t smem = (size_t)n_cols * 256 * sizeof(int4);
+  VX_TRY(raise_smem_limit(once, star_scan_kernel, 12 * 256 * sizeof(int4)));
   if (!occ) {
-    VX_CUDA_TRY(cudaFuncSetAttribute(star_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(12 * 256 * sizeof(int4))));
     VX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, star_scan_kernel, 256, 12 * 256 * sizeof(int4)));
     occ = std::max(occ, 1);
   }
@@ -1539,12 +1531,8 @@ struct StarExKernel : ExKernel {
       if (timed) VX_CUDA_TRY(rec(ev_b[ek]));
       const int gg = ctx->num_sms * 4;
       if (smem) {
-        static bool attr_g = false;
-        if (!attr_g) {
-          VX_CUDA_TRY(cudaFuncSetAttribute(star_gather_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(16 * kSmemGroups)));
-          attr_g = true;
-        }
+        static OncePerDevice once;
+        VX_TRY(raise_smem_limit(once, star_gather_kernel<true>, 16 * kSmemGroups));
         star_gather_kernel<true><<<gg, 256, smem_bytes, s>>>(p);
       } else {
         star_gather_kernel<false><<<gg, 256, 0, s>>>(p);
@@ -1575,23 +1563,15 @@ struct StarExKernel : ExKernel {
     } else if (ctx->cfg.kernel_rows == 16) {  // scalar kernel, 16 rows per thread
       g = grid_for(ctx, (p.n + 15) / 16, threads);
       if (smem) {
-        static bool attr16 = false;
-        if (!attr16) {
-          VX_CUDA_TRY(cudaFuncSetAttribute(star_chunk_kernel<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(16 * kSmemGroups)));
-          attr16 = true;
-        }
+        static OncePerDevice once;
+        VX_TRY(raise_smem_limit(once, star_chunk_kernel<true, 16>, 16 * kSmemGroups));
         star_chunk_kernel<true, 16><<<g, threads, smem_bytes, s>>>(p);
       } else {
         star_chunk_kernel<false, 16><<<g, threads, 0, s>>>(p);
       }
     } else if (smem) {
-      static bool attr_set = false;
-      if (!attr_set) {
-        VX_CUDA_TRY(cudaFuncSetAttribute(star_chunk_kernel<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(16 * kSmemGroups)));
-        attr_set = true;
-      }
+      static OncePerDevice once;
+      VX_TRY(raise_smem_limit(once, star_chunk_kernel<true, 8>, 16 * kSmemGroups));
       star_chunk_kernel<true, 8><<<g, threads, smem_bytes, s>>>(p);
     } else {
       star_chunk_kernel<false, 8><<<g, threads, 0, s>>>(p);
