@@ -112,11 +112,11 @@ struct TrainArgs {
 };
 
 // sigmoid of the training steps: the argument of exp stops at 80 (the result,
-// 2e-35, is far below what any sum keeps), so 1 + exp(-v) stays in the range
+// 2e-35, is far below what any sum keeps; a NaN stays one), so 1 + exp(-v) stays in the range
 // where the reciprocal needs no special case, and one Newton step takes the
 // approximate reciprocal to its last bit
 __device__ __forceinline__ float sigmoid_step(float v) {
-  const float d = 1.f + expf(fminf(-v, 80.f));
+  const float d = 1.f + expf(v < -80.f ? 80.f : -v);
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
   return fmaf(r, fmaf(-d, r, 1.f), r);
