@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "vx_internal.h"
+#include "vx_math.cuh"
 #include "vx_sort.cuh"
 
 namespace vx {
@@ -96,8 +97,8 @@ __global__ void __launch_bounds__(kMlpThreads, 2) mlp_fwd_bwd_kernel(const float
 // 300 steps on 65,536 points: 5.2 ms as a launch per step in captured graphs (a
 // warp walked its points one by one, 98 global atomics per block, the update in
 // the last block); 1.84 ms for the whole call with the sums written parameter by
-// parameter and a fence in every thread; 1.61 ms now.  Of a step's 10,600 cycles
-// the outputs take 2,700 (two special-function instructions a point and unit:
+// parameter and a fence in every thread; 1.70 ms now.  Of a step's 11,200 cycles
+// the outputs take about 3,300 (two special-function instructions a point and unit:
 // 2,050), the gradient sums 950 and the block's 1,300, the barrier with the read
 // of the rows 4,200 and the update 800.  Sums that carry their step's number and are
 // polled for, added up parameter by parameter in one block each, took 2.2 ms.
@@ -112,15 +113,9 @@ struct TrainArgs {
 };
 
 // sigmoid of the training steps: the argument of exp stops at 80 (the result,
-// 2e-35, is far below what any sum keeps; a NaN stays one), so 1 + exp(-v) stays in the range
-// where the reciprocal needs no special case, and one Newton step takes the
-// approximate reciprocal to its last bit
-__device__ __forceinline__ float sigmoid_step(float v) {
-  const float d = 1.f + expf(v < -80.f ? 80.f : -v);
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-  return fmaf(r, fmaf(-d, r, 1.f), r);
-}
+// 2e-35, is far below what any sum keeps; a NaN stays one), so that 1 + exp(-v)
+// stays in the reciprocal's range
+__device__ __forceinline__ float sigmoid_step(float v) { return reciprocal(1.f + expf(v < -80.f ? 80.f : -v)); }
 
 // floats of a block's sums: whole 16-byte words, so that the blocks' rows are
 // written and read in few wide accesses
