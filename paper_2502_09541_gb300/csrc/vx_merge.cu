@@ -705,7 +705,7 @@ struct MergePass : ExKernel {
   uint32_t *out_vals;
   int S;
   std::vector<int> result_buf;  // per slot: buffer holding the merged partition
-  uint64_t rounds_pairs = 0;
+  uint64_t rounds_pairs = 0, launches = 0;
   std::vector<cudaEvent_t> ev0, ev1;
   double ms_merge = 0;
   ~MergePass() override {
@@ -765,6 +765,7 @@ struct MergePass : ExKernel {
     VX_CUDA_TRY(cudaGetLastError());
     if (!ev1.empty()) VX_CUDA_TRY(cudaEventRecord(ev1[e], s));
     rounds_pairs += rounds * n;
+    launches += 2 * rounds;  // cuts and merge
     return VX_OK;
   }
   void on_retire(uint64_t p) override {
@@ -886,6 +887,7 @@ struct ResidentMergePass : MergePass {
     VX_CUDA_TRY(cudaGetLastError());
     if (!ev1.empty()) VX_CUDA_TRY(cudaEventRecord(ev1[e], s));
     rounds_pairs += rounds * seg.back();
+    launches += 2 * rounds;
     return VX_OK;
   }
   vx_status outputs(uint64_t p, char *slot, std::vector<CopyOp> &d2h) override {
@@ -908,7 +910,7 @@ struct TileMergePass : ExKernel {
   const uint32_t *d_cut;
   const uint64_t *d_rank;
   std::vector<uint64_t> rank;  // n_tiles + 1
-  uint64_t n, P, cap;
+  uint64_t n, P, cap, launches = 0;
   uint64_t *out_keys;
   uint32_t *out_vals;
   int S;
@@ -928,6 +930,7 @@ struct TileMergePass : ExKernel {
     tile_merge_kernel<<<t1 - t0, kTileThreads, sizeof(TileSmem), s>>>(runs, rk, rv, d_cut, d_rank, t0, o0, o1,
                                                                       (uint64_t *)slot, (uint32_t *)(slot + kb()));
     VX_CUDA_TRY(cudaGetLastError());
+    ++launches;
     return VX_OK;
   }
   bool has_outputs() override { return true; }
@@ -1069,7 +1072,7 @@ vx_status tile_merge(vx_ctx *ctx, const uint64_t *rk, const uint32_t *rv, uint64
   ExecStats es;
   VX_TRY(run_pipeline(ctx, mp, &es));
   ss.bytes_d2h += es.bytes_d2h;
-  ss.kernel_launches += es.kernel_launches + 15;
+  ss.kernel_launches += mp.launches + radix_launches() + 5;  // samples, their sort, home, publish, cuts, ranks
   ss.ms_merge_kernel += es.ms_kernel;
   ss.merge_pass_pairs += n;
   ss.slot_pairs = mp.cap;
@@ -1170,7 +1173,7 @@ vx_status resident_merge_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t 
     VX_TRY(run_pipeline(ctx, rp, &es));
     VX_CUDA_TRY(cudaStreamSynchronize(s));
     ss.bytes_h2d += es.bytes_h2d;
-    ss.kernel_launches += es.kernel_launches * 13;  // radix sort (10), home, fences, publish
+    ss.kernel_launches += es.kernel_launches * (radix_launches() + 3);  // and home, fences, publish
     ss.ms_sort_kernel += es.ms_kernel;
     ss.radix_pass_pairs += rp.pass_pairs;
     for (uint64_t at = 0; at < n; at += R) {
@@ -1226,7 +1229,7 @@ vx_status resident_merge_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t 
   ExecStats es;
   VX_TRY(run_pipeline(ctx, mp, &es));
   ss.bytes_d2h += es.bytes_d2h;
-  ss.kernel_launches += es.kernel_launches;
+  ss.kernel_launches += mp.launches;
   ss.ms_merge_kernel += mp.ms_merge;
   ss.merge_pass_pairs += mp.rounds_pairs;
   ss.slot_pairs = mp.cap;
@@ -1364,7 +1367,7 @@ vx_status merge_sort_plan(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
       VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
       ss.bytes_h2d += es.bytes_h2d;
       ss.bytes_d2h += es.bytes_d2h;
-      ss.kernel_launches += es.kernel_launches * 12;  // radix sort (10), fences, publish
+      ss.kernel_launches += es.kernel_launches * (radix_launches() + 2);  // and fences, publish
       ss.ms_sort_kernel += es.ms_kernel;
       ss.radix_pass_pairs += rp.pass_pairs;
     }
@@ -1440,7 +1443,7 @@ vx_status merge_sort_plan(vx_ctx *ctx, const uint64_t *keys, const uint32_t *val
   VX_TRY(run_pipeline(ctx, mp, &es));
   ss.bytes_h2d += es.bytes_h2d;
   ss.bytes_d2h += es.bytes_d2h;
-  ss.kernel_launches += es.kernel_launches;
+  ss.kernel_launches += mp.launches;
   ss.ms_merge_kernel += mp.ms_merge;
   ss.merge_pass_pairs += mp.rounds_pairs;
   ss.slot_pairs = mp.cap;

@@ -720,7 +720,7 @@ vx_status radix_join_resident(vx_ctx *ctx, const Column *bk, const Column *bp, c
         pp.mid_keys, n, R, (1ull << bits) - 1, run_shift, n_runs, (uint32_t *)(m + (side ? rs.bbnd : rs.abnd)));
     VX_CUDA_TRY(cudaGetLastError());
     res.bytes_h2d += es.bytes_h2d;
-    res.kernel_launches += es.kernel_launches * (pp.npass - pp.first + 3) + 1;
+    res.kernel_launches += es.kernel_launches * (radix_launches(pp.npass, pp.first) + 1) + 1;  // keep; cuts
     res.ms_kernel += es.ms_kernel;
   }
   res.ms_partition = res.ms_build = now_ms() - tp;
@@ -876,7 +876,8 @@ vx_status radix_join(vx_ctx *ctx, const Column *bk, const Column *bp, const Colu
     VX_TRY(run_pipeline(ctx, pp, &es));
     res.bytes_h2d += es.bytes_h2d;
     res.bytes_d2h += es.bytes_d2h;
-    res.kernel_launches += es.kernel_launches * (npass + 9);
+    // rows, the sort, boundaries (4), publish, and the build side's payloads
+    res.kernel_launches += es.kernel_launches * (radix_launches(npass) + 6 + (pp.payload ? 1 : 0));
     res.ms_kernel += es.ms_kernel;
   }
   res.ms_partition = now_ms() - tp;
@@ -982,7 +983,7 @@ vx_status radix_join(vx_ctx *ctx, const Column *bk, const Column *bp, const Colu
     ExecStats es;
     VX_TRY(run_pipeline(ctx, jp, &es));
     res.bytes_h2d += es.bytes_h2d;
-    res.kernel_launches += es.kernel_launches;
+    res.kernel_launches += es.kernel_launches * 2;  // work items and join
     res.ms_kernel += jp.ms_join;
     res.ms_probe_kernel = jp.ms_join;
   }

@@ -1371,7 +1371,7 @@ struct ResidentSortPass : ExKernel {
   uint32_t *out_vals;
   int S;
   int first;  // sort by the key bytes first .. 7 and repair, 0: by all
-  uint64_t pass_pairs = 0;
+  uint64_t pass_pairs = 0, launches = 0;
   uint64_t size() override { return jobs.size(); }
   int n_slots() override { return S; }
   int max_in_flight() override { return S; }
@@ -1395,6 +1395,7 @@ struct ResidentSortPass : ExKernel {
       VX_TRY(radix_prefix_sort_enqueue(bufs(j, slot), j.n, temp, s, ctx->num_sms, first, ctx->cfg.lookback_spin_limit));
     else
       VX_TRY(radix_sort_enqueue(bufs(j, slot), j.n, temp, s, ctx->num_sms, 8, ctx->cfg.lookback_spin_limit));
+    launches += (first ? radix_prefix_launches(j.n, first) : radix_launches()) + 1;  // and publish
     return radix_publish_enqueue(temp, ctx->d_scalars + 64 + (it % S), s);
   }
   bool has_outputs() override { return true; }
@@ -1419,6 +1420,7 @@ struct ResidentSortPass : ExKernel {
         char *temp = slot + kb() + vb();
         VX_TRY(radix_sort_enqueue(b, j.n, temp, ctx->s_compute, ctx->num_sms, 8, ctx->cfg.lookback_spin_limit));
         VX_TRY(radix_publish_enqueue(temp, ctx->d_scalars + 64 + (it % S), ctx->s_compute));
+        launches += radix_launches() + 1;
         VX_CUDA_TRY(cudaStreamSynchronize(ctx->s_compute));
       }
     }
@@ -1604,7 +1606,7 @@ vx_status resident_sort(vx_ctx *ctx, const uint64_t *keys, const uint32_t *vals,
   VX_TRY(run_pipeline(ctx, sp, &es));
   ss.bytes_h2d += es.bytes_h2d;
   ss.bytes_d2h += es.bytes_d2h;
-  ss.kernel_launches += es.kernel_launches * 11;  // byte histogram, state, 8 passes, publish
+  ss.kernel_launches += sp.launches;
   ss.ms_sort_kernel += es.ms_kernel;
   ss.radix_pass_pairs += sp.pass_pairs;
   ss.ms_sort += now_ms() - t0;
@@ -1651,7 +1653,7 @@ static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *v
     VX_TRY(run_pipeline(ctx, sp, &es));
     ss.bytes_h2d += es.bytes_h2d;
     ss.bytes_d2h += es.bytes_d2h;
-    ss.kernel_launches += es.kernel_launches;
+    ss.kernel_launches += es.kernel_launches * (radix_launches() + 1);  // and publish
     ss.ms_sort_kernel += es.ms_kernel;
     ss.radix_pass_pairs += sp.pass_pairs;
     ss.n_partitions = std::max<uint32_t>(ss.n_partitions, 1);
@@ -1913,7 +1915,7 @@ static vx_status sort_pairs(vx_ctx *ctx, const uint64_t *keys, const uint32_t *v
     VX_TRY(run_pipeline(ctx, sp, &es));
     ss.bytes_h2d += es.bytes_h2d;
     ss.bytes_d2h += es.bytes_d2h;
-    ss.kernel_launches += es.kernel_launches * 11;  // byte histogram, state, 8 passes, publish
+    ss.kernel_launches += es.kernel_launches * (radix_launches() + 1);  // and publish
     ss.ms_sort_kernel += es.ms_kernel;
     ss.radix_pass_pairs += sp.pass_pairs;
   }

@@ -29,6 +29,12 @@ vx_status radix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s
 // stable rearrangement of the input) have to be sorted in full.
 vx_status radix_prefix_sort_enqueue(RadixBufs b, uint64_t n, char *temp, cudaStream_t s, int num_sms, int first,
                                     uint32_t spin_limit, cudaEvent_t vals = nullptr);
+// Kernels that a sort enqueues: the histogram and the digits' bases, then a
+// scatter per key byte, and for a prefix sort the search and the repair
+constexpr uint64_t radix_launches(int npass = 8, int first = 0) { return (uint64_t)(npass - first) + 2; }
+constexpr uint64_t radix_prefix_launches(uint64_t n, int first) {
+  return n < 2 || n >> 32 ? radix_launches() : radix_launches(8, first) + 2;
+}
 // after radix_sort_enqueue on s: publishes to a mapped host word the buffer
 // holding the result (low byte), the executed passes (next byte), whether
 // a look-back wait gave up (bit 16) and the prefix sort's bit 17
