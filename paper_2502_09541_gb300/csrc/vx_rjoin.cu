@@ -830,7 +830,7 @@ vx_status radix_join(vx_ctx *ctx, const Column *bk, const Column *bp, const Colu
   int run_bits = 0;
   while (run_bits < bits && run_bits < 20 && (nb >> run_bits) > kRjRunBuild) ++run_bits;
   const int run_shift = bits - run_bits;
-  const uint32_t step = 1u << run_shift;
+  uint32_t step = 1u << run_shift;
 
   // ---- both clustered tables in the arena, if they fit beside the slots of
   // the partition pass (chunks small enough to pipeline)
@@ -892,6 +892,27 @@ vx_status radix_join(vx_ctx *ctx, const Column *bk, const Column *bp, const Colu
     for (uint32_t c = 0; c < N; ++c) t += bnd[c * G1 + g];
     return t;
   };
+  // Build keys may crowd into a small part of the groups (dense small keys do),
+  // and runs of more tuples than a table takes read their probe tuples once per
+  // table: shorter runs, as long as they make the run that a build tuple is in
+  // smaller.  200M probes of 200,000 dense keys: join kernel 20.7 -> 1.1 ms; of
+  // 700,000 13.0 -> 1.2.  Uniform keys keep their runs.
+  auto run_size = [&](uint32_t groups) {
+    double squares = 0;
+    uint64_t below = 0;
+    for (uint64_t g = groups; g <= G && nb; g += groups) {
+      const uint64_t t = tuples_below(abnd, NA, g);
+      squares += (double)(t - below) * (double)(t - below);
+      below = t;
+    }
+    return nb ? squares / (double)nb : 0.0;
+  };
+  for (double size = run_size(step); step > 1 && size > kRjPiece;) {
+    const double half = run_size(step / 2);
+    if (half > 0.75 * size) break;  // one group's tuples
+    step /= 2;
+    size = half;
+  }
   const uint64_t slot_b = (uint64_t)((double)ctx->arena.largest_free() / S * 0.95) / 256 * 256;
   auto layout = [&](RjRange &r) {
     const uint64_t ng1 = r.g1 - r.g0 + 1;
