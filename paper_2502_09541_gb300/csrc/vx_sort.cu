@@ -2053,8 +2053,12 @@ VX_API vx_status vx_radix_sort_pairs(vx_ctx *ctx, const uint64_t *keys, const ui
   } vals_in{ctx->s_h2d};
   if (sample) {
     VX_CUDA_TRY(cudaEventCreateWithFlags(&vals_in.e, cudaEventDisableTiming));
-    VX_CUDA_TRY(cudaEventRecord(vals_in.e, s));
-    VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_h2d, vals_in.e, 0));
+    const cudaError_t idle = cudaStreamQuery(s);
+    if (idle != cudaSuccess) {  // work left; where there is none, asking costs 2 us of a call and the wait up to 7
+      if (idle != cudaErrorNotReady) VX_CUDA_TRY(idle);
+      VX_CUDA_TRY(cudaEventRecord(vals_in.e, s));
+      VX_CUDA_TRY(cudaStreamWaitEvent(ctx->s_h2d, vals_in.e, 0));
+    }
   }
   VX_CUDA_TRY(cudaMemcpyAsync(b.keys[0], keys, 8 * n, cudaMemcpyHostToDevice, s));
   volatile uint64_t *word = ctx->h_scalars + 64;
