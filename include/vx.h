@@ -177,8 +177,8 @@ vx_status vx_filter(vx_ctx *ctx, const vx_pred *preds, int32_t n_preds, uint64_t
  * behaviour:
  *   - n_rows above 67,108,864 (2^26) returns VX_E_INVAL;
  *   - count > cap returns VX_E_CAPACITY after writing the first cap ids;
- *   - the call's blocks wait for one another's counts; a wait that runs out
- *     (each is bounded) returns VX_E_TIMEOUT;
+ *   - the call's blocks wait for one another's counts, each only for blocks that
+ *     have started; a wait that runs out (each is bounded) returns VX_E_TIMEOUT;
  *   - the first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress with that device current) and keeps it for the
  *     life of the process, so the device must not be reset (cudaDeviceReset)
@@ -374,7 +374,12 @@ enum { VX_SORT_PARTITION = 0, VX_SORT_MERGE = 1 };
 
 typedef struct {
   int32_t partitioner;        /* VX_PART_*: how the range partition's splitters are chosen */
-  int32_t n_partitions;       /* 0 = smallest count whose expected partition fits a slot; <= 256 */
+  int32_t n_partitions;       /* 0 = from the arena and the input.  Where the pairs stay in the arena
+                                 (see vx_sort): PARTITION, n / 12e6 rounded up, more where two slots
+                                 of the second pass need it, 4 to 64; MERGE, n / 2^22, at most 64, or
+                                 as many as its slots need.  Else the smallest count whose expected
+                                 partition fits a slot, with headroom, and at least 16 for large inputs.
+                                 At most 128 (PARTITION).  stats->n_partitions is what resulted */
   uint64_t seed;              /* sample positions */
   uint64_t sample_size;       /* keys sampled for the splitters (0 = 1 Mi) */
   uint32_t mlp_steps;         /* Adam steps of the CDF MLP (0 = 300) */
@@ -390,7 +395,9 @@ typedef struct {
                                  bytes (stats: contiguous_layout) */
   uint64_t host_scratch_bytes;
   uint64_t max_slot_pairs;    /* optional cap on the pairs per staging slot (0 = from the arena) */
-  uint64_t *splitters_out;    /* optional: receives the P-1 top-level splitters (PARTITION plan) */
+  uint64_t *splitters_out;    /* optional: receives the stats->n_partitions - 1 top-level splitters
+                                 (PARTITION plan); room for 2 (n_partitions - 1) values, or 254 with
+                                 n_partitions 0 */
   int32_t plan;               /* VX_SORT_PARTITION (default) or VX_SORT_MERGE */
   int32_t runs_mode;          /* MERGE: 0 = when a sample of adjacent pairs suggests the input is
                                  made of at most 256 ascending runs, find them (one pass over the
@@ -406,7 +413,9 @@ typedef struct {
   uint64_t max_partition, min_partition, slot_pairs;
   double imbalance;                /* largest partition / mean partition */
   double ms_sample, ms_train, ms_partition, ms_sort, ms_total;
-  uint64_t bytes_h2d, bytes_d2h, kernel_launches;
+  uint64_t bytes_h2d, bytes_d2h;
+  uint64_t kernel_launches;        /* kernels of the passes' chunks, partitions and runs (not the sample's
+                                      and the splitters') */
   double ms_sort_kernel;           /* device time of the per-partition radix sorts (CUDA events) */
   uint64_t radix_pass_pairs;       /* pairs x executed LSD passes in those sorts (skipped digits excluded) */
   uint64_t out_of_region_pairs;    /* pairs stored past their partition's region (overflow area,

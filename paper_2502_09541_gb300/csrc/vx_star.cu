@@ -837,8 +837,9 @@ __global__ void __launch_bounds__(256) star_split_kernel(const ChunkParams p) {
 // mapped host memory with one independent load per survivor in flight, and
 // aggregated into the group accumulators.  A chunk whose survivors did not
 // fit the list is not aggregated at all: it is flagged for an exact rerun.
-// A plan without group keys has one accumulator: each block adds its total to it
-// once.  (A 64-bit shared-memory add per survivor made the block's survivors
+// A plan without group keys has one accumulator: each warp adds its total once, to
+// its block's word (added to the plan's at the end) or, without shared-memory
+// accumulators, to the plan's.  (A 64-bit shared-memory add per survivor made the block's survivors
 // queue for one word: 30 us a chunk of 9,300 survivors beside the next chunk's
 // copy, 13 now.)
 template <bool kSmem>

@@ -160,11 +160,11 @@ __device__ __forceinline__ void sf_scan_block(const SfParams &p, volatile uint64
 // does nothing but turn the tiles' counts into prefixes; then the survivors leave
 // as one contiguous run.  The scan block works on whole windows, whose later
 // tiles may not have a place on the GPU yet, so a tile whose prefix does not come
-// looks back itself: no tile needs one that has not started.  Three columns of 2^26 rows, 2 % qualifying: 171 us
-// for the call, of which 20 us are not the kernel (5.4 TB/s, 0.79 of the
-// measured copy bandwidth); 907 us when a count pass, a scan of the tiles and a
-// write pass read the columns twice in 4-byte loads.  10,007 rows, two columns:
-// 21 us, 42 us before.
+// looks back itself: no tile needs one that has not started.  Three columns of
+// 2^26 rows, 2 % qualifying: 171 us for the call, of which 20 us are not the
+// kernel (5.4 TB/s, 0.79 of the measured copy bandwidth); 907 us when a count pass,
+// a scan of the tiles and a write pass read the columns twice in 4-byte loads.
+// 10,007 rows, two columns: 21 us, 42 us before.
 template <bool kVec, int kG, bool kScan>
 __global__ void __launch_bounds__(kSfThreads) sf_filter_kernel(const SfParams p, uint32_t *scratch, uint64_t *out) {
   constexpr int kB = kG / 4;  // batches of four groups

@@ -15,7 +15,7 @@ static __device__ unsigned long long now_ns() {
 __global__ void hold(unsigned long long ns, unsigned int *started) {
   const unsigned long long t0 = now_ns();
   atomicAdd_system(started, 1u);
-  for (int i = 0; i < 100000000 && now_ns() - t0 < ns; ++i) __nanosleep(10000);
+  for (unsigned long long i = 0; i < ns / 1000 && now_ns() - t0 < ns; ++i) __nanosleep(10000);
 }
 
 static cudaStream_t g_stream;
